@@ -175,6 +175,63 @@ constexpr int kBlobSmall = 1024;
 constexpr int kBlobMid = 8192;
 constexpr int kBlobLarge = 31 * 1024;  // header + blob stays below the 32,764-byte parameter limit
 
+// ---- tiled launches (see tile_copy): the segments cut into 16 KiB tiles,
+// one CTA each. 512 threads x 2 vectors, from a sweep on GB300 (us a pass;
+// put + get of B=4 requests of 45 MB on one stream / of 16 B=8 requests of
+// 92 MB on four / get of 2.7 GB / put, compaction and get of 1 GiB): 512 x 2
+// 94.1 / 810 / 755 / 895; 1024 x 2 94.6 / 810 / 765 / 901; 512 x 4 98.2 / 814 /
+// 759 / 904; 256 x 4 96.7 / 815 / 760 / 904; 256 x 2 95.1 / 812 / 757 / 900;
+// 128 x 4 93.9 / 815 / 760 / 904. Without the L2 prefetch: 102.0 / 811 / 757 / 902.
+#ifndef T2I_TUNE_TILE_THREADS
+#define T2I_TUNE_TILE_THREADS 512
+#endif
+#ifndef T2I_TUNE_TILE_VEC
+#define T2I_TUNE_TILE_VEC 2
+#endif
+#ifndef T2I_TUNE_TILE_BLOCKS
+#define T2I_TUNE_TILE_BLOCKS 4
+#endif
+#ifndef T2I_TUNE_TILE_MIN_BYTES
+#define T2I_TUNE_TILE_MIN_BYTES (4ull << 20)
+#endif
+constexpr int kTileThreads = T2I_TUNE_TILE_THREADS;
+constexpr int kTileVec = T2I_TUNE_TILE_VEC;
+constexpr uint32_t kTileBytes = kTileThreads * kTileVec * 16;  // 16 KiB
+constexpr uint32_t kTileShift = kTileBytes == 8192 ? 13 : kTileBytes == 16384 ? 14 : kTileBytes == 32768 ? 15 : 16;
+static_assert(kTileBytes == 1u << kTileShift, "tile size");
+// Aligned launches of at least this many bytes run as tiles. Below it the
+// launch is bound by its latency, and the other kernels' 16 KiB shares are
+// the same size: eight B=1 requests (11.5 MB a call) took 89.3 us a pass in
+// those kernels and 69 in tiles, a 16 MiB get the same in both.
+constexpr uint64_t kTileMinBytes = T2I_TUNE_TILE_MIN_BYTES;
+
+struct TileSeg {
+    uint64_t user;
+    uint32_t nbytes;  // 1 .. 1 GiB: longer segments are split at page boundaries
+    uint32_t tile0;   // first tile of the segment in the launch
+    uint32_t page;    // its page number (kTileOnePage), else its first entry in the page array
+    uint32_t flags;
+};
+static_assert(sizeof(TileSeg) == 24, "TileSeg layout");
+constexpr uint32_t kTileCast = 1u;     // fp32 -> bf16 (get only)
+constexpr uint32_t kTileOnePage = 2u;  // one page, or a run of consecutive ones from `page` on
+constexpr uint64_t kTileMaxSegBytes = uint64_t(1) << 30;
+
+struct TileHeader {
+    uint64_t pool;
+    uint32_t n_seg;
+    uint32_t page_shift;
+    uint32_t pages_offset;  // byte offset of the uint32 page array in blob
+    uint32_t flags;         // kPrefetchSources, or 0
+};
+static_assert(sizeof(TileHeader) == 24, "TileHeader layout");
+
+template <int BLOB>
+struct TileParams {
+    TileHeader h;
+    alignas(8) unsigned char blob[BLOB];  // TileSeg[n_seg], then uint32 pages[]
+};
+
 // GetCopy: a get whose launch has no cast segment (a leaner kernel).
 enum class Mode { Put, Get, Move, GetCopy };
 
@@ -638,6 +695,62 @@ __device__ __forceinline__ void prefetch_share(const LaunchParams<BLOB>& p) {
         asm volatile("prefetch.global.L2 [%0];" ::"l"(first + (uint64_t(k) << 7)));
 }
 
+// The copy of one tile (len <= kTileBytes, both sides 16-byte aligned).
+__device__ __forceinline__ void tile_copy_bytes(unsigned char* __restrict__ dst, const unsigned char* __restrict__ src,
+                                                uint32_t len) {
+    const uint32_t nvec = len >> 4;
+    const uint4* s = reinterpret_cast<const uint4*>(src);
+    uint4* d = reinterpret_cast<uint4*>(dst);
+    uint4 r[kTileVec];
+#pragma unroll
+    for (int j = 0; j < kTileVec; ++j) {
+        const uint32_t v = j * kTileThreads + threadIdx.x;
+        if (v < nvec) r[j] = ld_stream(s + v);
+    }
+#pragma unroll
+    for (int j = 0; j < kTileVec; ++j) {
+        const uint32_t v = j * kTileThreads + threadIdx.x;
+        if (v < nvec) st_stream(d + v, r[j]);
+    }
+    const uint32_t at = (nvec << 4) + threadIdx.x;
+    if (at < len) dst[at] = src[at];
+}
+
+// The same with the cast: len source bytes, a multiple of 4. Blocks of 8
+// floats (two 16-byte loads, one 16-byte store), the last < 8 one by one.
+__device__ __forceinline__ void tile_cast(unsigned char* __restrict__ dst, const unsigned char* __restrict__ src,
+                                          uint32_t len) {
+    static_assert(kTileVec % 2 == 0, "a block is two vectors");
+    const uint32_t n8 = len >> 5;
+    const uint4* s = reinterpret_cast<const uint4*>(src);
+    uint4* d = reinterpret_cast<uint4*>(dst);
+    constexpr int kSteps = kTileVec / 2;
+    uint4 a[kSteps], b[kSteps];
+#pragma unroll
+    for (int j = 0; j < kSteps; ++j) {
+        const uint32_t v = j * kTileThreads + threadIdx.x;
+        if (v < n8) {
+            a[j] = ld_stream(s + 2 * v);
+            b[j] = ld_stream(s + 2 * v + 1);
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < kSteps; ++j) {
+        const uint32_t v = j * kTileThreads + threadIdx.x;
+        if (v < n8) {
+            uint4 o;
+            o.x = pack_bf16x2(a[j].x, a[j].y);
+            o.y = pack_bf16x2(a[j].z, a[j].w);
+            o.z = pack_bf16x2(b[j].x, b[j].y);
+            o.w = pack_bf16x2(b[j].z, b[j].w);
+            st_stream(d + v, o);
+        }
+    }
+    const uint32_t at = (n8 << 3) + threadIdx.x;
+    if (at < len >> 2)
+        reinterpret_cast<uint16_t*>(dst)[at] = (uint16_t)bf16_rne_bits(reinterpret_cast<const uint32_t*>(src)[at]);
+}
+
 // Programmatic dependent launch: wait until the previous grid in the stream
 // has completed and its memory is visible (returns at once when this launch
 // has no such dependency), then let the next launch begin its set-up.
@@ -776,6 +889,53 @@ __device__ __forceinline__ void run_range(const LaunchParams<BLOB>& p, uint64_t 
     }
 }
 
+// ------------------------------------------------------------- tiled launches
+// One CTA per tile: the 16 KiB (or the rest) of one segment at a multiple of
+// 16 KiB, in one page or one run of pages, both sides 16-byte aligned. Bound
+// by HBM; between launches on one stream by the drain of one grid and the
+// ramp-up of the next. So a CTA lives for one round of straight-line code:
+// its tile is worked out, and its source lines asked of L2, before the wait
+// for the previous grid; then come its loads, then its stores. CTAs of the
+// next grid take over an SM 16 KiB at a time as this one drains, and the
+// hardware block scheduler balances the SMs without a counter or a barrier.
+// Against CTAs that walk 64 KiB shares in 32 KiB rounds (us a pass, the cases
+// of the sweep above): 109.9 / 818 / 766 / 921; requests pulled between
+// stores (92 MB a launch) 54.7 -> 51.8.
+template <Mode M, int BLOB>
+__device__ __forceinline__ void tile_copy(const TileParams<BLOB>& p) {
+    constexpr bool kToUser = M == Mode::Get;
+    const TileSeg* segs = reinterpret_cast<const TileSeg*>(p.blob);
+    uint32_t lo = 0, hi = p.h.n_seg - 1;
+    while (lo < hi) {  // the last segment that starts at or before this tile
+        const uint32_t mid = (lo + hi + 1) >> 1;
+        if (segs[mid].tile0 <= blockIdx.x)
+            lo = mid;
+        else
+            hi = mid - 1;
+    }
+    const uint32_t off = (blockIdx.x - segs[lo].tile0) << kTileShift;
+    const uint32_t len = umin(kTileBytes, segs[lo].nbytes - off);
+    const uint32_t flags = segs[lo].flags;
+    const bool cast = kToUser && (flags & kTileCast);
+    uint32_t page = segs[lo].page, in_page = off;
+    if (!(flags & kTileOnePage)) {
+        const uint32_t* pages = reinterpret_cast<const uint32_t*>(p.blob + p.h.pages_offset);
+        page = pages[page + (off >> p.h.page_shift)];
+        in_page = off & ((1u << p.h.page_shift) - 1);
+    }
+    unsigned char* pa = reinterpret_cast<unsigned char*>(p.h.pool) + (uint64_t(page) << p.h.page_shift) + in_page;
+    unsigned char* ua = reinterpret_cast<unsigned char*>(segs[lo].user) + (cast ? off >> 1 : off);
+    const unsigned char* src = kToUser ? pa : ua;
+    unsigned char* dst = kToUser ? ua : pa;
+    if (kPrefetch && (p.h.flags & kPrefetchSources) && threadIdx.x * 128u < len)
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(src + threadIdx.x * 128u));
+    pdl_wait_then_release();
+    if (cast)
+        tile_cast(dst, src, len);
+    else
+        tile_copy_bytes(dst, src, len);
+}
+
 // Named entry points (one per operation, so that profiles name them).
 template <int BLOB, bool GENERAL>
 __global__ void __launch_bounds__(kThreads, GENERAL ? kMinBlocksGeneral : kMinBlocks)
@@ -799,6 +959,21 @@ __global__ void __launch_bounds__(kThreads, GENERAL ? kMinBlocksGeneral : kMinBl
     prefetch_share<Mode::GetCopy, BLOB>(p);
     pdl_wait_then_release();
     run_share<Mode::GetCopy, GENERAL, BLOB>(p);
+}
+template <int BLOB>
+__global__ void __launch_bounds__(kTileThreads, T2I_TUNE_TILE_BLOCKS)
+    put_tile_kernel(const __grid_constant__ TileParams<BLOB> p) {
+    tile_copy<Mode::Put, BLOB>(p);
+}
+template <int BLOB>
+__global__ void __launch_bounds__(kTileThreads, T2I_TUNE_TILE_BLOCKS)
+    get_tile_kernel(const __grid_constant__ TileParams<BLOB> p) {
+    tile_copy<Mode::Get, BLOB>(p);
+}
+template <int BLOB>
+__global__ void __launch_bounds__(kTileThreads, T2I_TUNE_TILE_BLOCKS)
+    move_tile_kernel(const __grid_constant__ TileParams<BLOB> p) {
+    tile_copy<Mode::Move, BLOB>(p);
 }
 template <int BLOB>
 __global__ void __launch_bounds__(kThreads, kMinBlocks) compact_move_kernel(const __grid_constant__ LaunchParams<BLOB> p) {

@@ -8,6 +8,32 @@
 // namespace t2i.
 #pragma once
 
+// One kernel launch of the parameters in param_buf_.
+inline t2i_status Store::launch_kernel(const void* fn, unsigned grid, unsigned threads, cudaStream_t stream) {
+    void* args[] = {param_buf_};
+    if (fail_countdown_ && --fail_countdown_ == 0) {
+        err_ = "kernel launch failed: injected failure (t2i_inject_launch_failure)";
+        return T2I_ERR_CUDA;
+    }
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3(grid);
+    lc.blockDim = dim3(threads);
+    lc.dynamicSmemBytes = 0;
+    lc.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    lc.attrs = attr;
+    lc.numAttrs = 1;
+    cudaError_t e = cudaLaunchKernelExC(&lc, fn, args);
+    if (e != cudaSuccess) {
+        err_ = std::string("kernel launch failed: ") + cudaGetErrorString(e);
+        return T2I_ERR_CUDA;
+    }
+    ctl_.counters().launches++;
+    return T2I_OK;
+}
+
 template <Mode M, bool GENERAL, int BLOB>
 t2i_status Store::launch_one(const std::vector<SegDesc>& sd, const std::vector<uint32_t>& pages, uint32_t n_granules,
                              cudaStream_t stream) {
@@ -49,32 +75,94 @@ t2i_status Store::launch_one(const std::vector<SegDesc>& sd, const std::vector<u
                                                                      0x7FFFFFFFull));
     const unsigned grid = static_cast<unsigned>(g);
     p->h.prefetch_ctas = kPrefetchFirstWave ? static_cast<uint32_t>(std::min<uint64_t>(g, resident)) : grid;
-    void* args[] = {p};
     const void* fn = M == Mode::Put                  ? reinterpret_cast<const void*>(scatter_put_kernel<BLOB, GENERAL>)
                      : mode == int(Mode::GetCopy)     ? reinterpret_cast<const void*>(gather_copy_kernel<BLOB, GENERAL>)
                      : M == Mode::Get                 ? reinterpret_cast<const void*>(gather_get_kernel<BLOB, GENERAL>)
                                                       : reinterpret_cast<const void*>(compact_move_kernel<BLOB>);
-    if (fail_countdown_ && --fail_countdown_ == 0) {
-        err_ = "kernel launch failed: injected failure (t2i_inject_launch_failure)";
-        return T2I_ERR_CUDA;
+    return launch_kernel(fn, grid, kThreads, stream);
+}
+
+template <Mode M, int BLOB>
+t2i_status Store::launch_tiles_one(uint32_t n_tiles, cudaStream_t stream) {
+    auto* p = reinterpret_cast<TileParams<BLOB>*>(param_buf_);
+    p->h.pool = pool_;
+    p->h.n_seg = static_cast<uint32_t>(ts_.size());
+    p->h.page_shift = page_shift_;
+    p->h.pages_offset = static_cast<uint32_t>(ts_.size() * sizeof(TileSeg));
+    p->h.flags = launch_flags_;
+    std::memcpy(p->blob, ts_.data(), ts_.size() * sizeof(TileSeg));
+    std::memcpy(p->blob + p->h.pages_offset, lp_.data(), lp_.size() * sizeof(uint32_t));
+    const void* fn = M == Mode::Put   ? reinterpret_cast<const void*>(put_tile_kernel<BLOB>)
+                     : M == Mode::Get ? reinterpret_cast<const void*>(get_tile_kernel<BLOB>)
+                                      : reinterpret_cast<const void*>(move_tile_kernel<BLOB>);
+    return launch_kernel(fn, n_tiles, kTileThreads, stream);
+}
+
+// Every user address of `segs` is 16-byte aligned.
+template <Mode M>
+t2i_status Store::launch_tiles(const std::vector<Seg>& segs, cudaStream_t stream) {
+    ts_.clear();
+    lp_.clear();
+    uint32_t tiles = 0;
+    auto flush = [&]() -> t2i_status {
+        if (ts_.empty()) return T2I_OK;
+        const size_t bytes = ts_.size() * sizeof(TileSeg) + lp_.size() * sizeof(uint32_t);
+        const t2i_status st = bytes <= size_t(kBlobTiny)    ? launch_tiles_one<M, kBlobTiny>(tiles, stream)
+                              : bytes <= size_t(kBlobSmall) ? launch_tiles_one<M, kBlobSmall>(tiles, stream)
+                              : bytes <= size_t(kBlobMid)   ? launch_tiles_one<M, kBlobMid>(tiles, stream)
+                                                            : launch_tiles_one<M, kBlobLarge>(tiles, stream);
+        ts_.clear();
+        lp_.clear();
+        tiles = 0;
+        return st;
+    };
+    const uint64_t P = uint64_t(1) << page_shift_;
+    const uint64_t max_pages = (kBlobLarge - sizeof(TileSeg)) / sizeof(uint32_t);
+    for (const Seg& s : segs) {
+        const uint64_t nbytes = s.nbytes_flags & kSegBytesMask;
+        const bool cast = (s.nbytes_flags & kCastFlag) != 0;
+        const bool run = pages_are_run(s);
+        const uint64_t step = run ? kTileMaxSegBytes / P : std::min<uint64_t>(kTileMaxSegBytes / P, max_pages);
+        for (uint64_t p0 = 0; p0 < s.n_pages; p0 += step) {
+            const uint64_t np = std::min<uint64_t>(step, s.n_pages - p0);
+            const bool one = run || np == 1;
+            const uint64_t off = p0 * P;
+            const uint64_t seg_bytes = std::min<uint64_t>(nbytes - off, np * P);
+            const size_t need = (ts_.size() + 1) * sizeof(TileSeg) + (lp_.size() + (one ? 0 : np)) * sizeof(uint32_t);
+            const uint64_t seg_tiles = (seg_bytes + kTileBytes - 1) / kTileBytes;
+            if (need > size_t(kBlobLarge) || tiles + seg_tiles > 0x7FFFFFFFull) {
+                t2i_status st = flush();
+                if (st != T2I_OK) return st;
+            }
+            TileSeg d;
+            d.user = s.user + (cast ? off / 2 : off);
+            d.nbytes = static_cast<uint32_t>(seg_bytes);
+            d.tile0 = tiles;
+            d.page = one ? s.pages[p0] : static_cast<uint32_t>(lp_.size());
+            d.flags = (cast ? kTileCast : 0) | (one ? kTileOnePage : 0);
+            ts_.push_back(d);
+            if (!one) lp_.insert(lp_.end(), s.pages + p0, s.pages + p0 + np);
+            tiles += static_cast<uint32_t>(seg_tiles);
+        }
     }
-    cudaLaunchConfig_t lc = {};
-    lc.gridDim = dim3(grid);
-    lc.blockDim = dim3(kThreads);
-    lc.dynamicSmemBytes = 0;
-    lc.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    lc.attrs = attr;
-    lc.numAttrs = 1;
-    cudaError_t e = cudaLaunchKernelExC(&lc, fn, args);
-    if (e != cudaSuccess) {
-        err_ = std::string("kernel launch failed: ") + cudaGetErrorString(e);
-        return T2I_ERR_CUDA;
+    return flush();
+}
+
+// Whether an aligned launch runs as tiles: it is large enough, its segments
+// fill their last tiles well enough (half-empty tiles cost as much to launch
+// as full ones), and every tile lies in one page or run.
+bool Store::tiles_fit(const std::vector<Seg>& segs) const {
+    uint64_t bytes = 0, tiles = 0;
+    for (const Seg& s : segs) {
+        const uint64_t n = s.nbytes_flags & kSegBytesMask;
+        bytes += n;
+        tiles += (n + kTileBytes - 1) / kTileBytes;
     }
-    ctl_.counters().launches++;
-    return T2I_OK;
+    if (bytes < kTileMinBytes || tiles * kTileBytes > bytes + bytes / 4) return false;
+    if (page_shift_ >= kTileShift) return true;
+    for (const Seg& s : segs)
+        if (!pages_are_run(s)) return false;
+    return true;
 }
 
 // Segments whose user address is 16-byte aligned go to the aligned kernels,
@@ -85,7 +173,8 @@ t2i_status Store::launch_segments(const std::vector<Seg>& segs, cudaStream_t str
     general_.clear();
     for (const Seg& s : segs) ((s.user & 15u) == 0 ? aligned_ : general_).push_back(s);
     t2i_status st = T2I_OK;
-    if (!aligned_.empty()) st = launch_group<M, false>(aligned_, stream);
+    if (!aligned_.empty())
+        st = tiles_fit(aligned_) ? launch_tiles<M>(aligned_, stream) : launch_group<M, false>(aligned_, stream);
     if (st == T2I_OK && !general_.empty()) {
         if (M == Mode::Move) return T2I_ERR_INVALID;  // pool pages are always aligned
         st = launch_group<(M == Mode::Move ? Mode::Put : M), true>(general_, stream);

@@ -212,6 +212,17 @@ class Store {
     template <Mode M, bool GENERAL, int BLOB>
     t2i_status launch_one(const std::vector<SegDesc>& sd, const std::vector<uint32_t>& pages, uint32_t n_granules,
                           cudaStream_t stream);
+    t2i_status launch_kernel(const void* fn, unsigned grid, unsigned threads, cudaStream_t stream);
+    template <Mode M>
+    t2i_status launch_tiles(const std::vector<Seg>& segs, cudaStream_t stream);
+    template <Mode M, int BLOB>
+    t2i_status launch_tiles_one(uint32_t n_tiles, cudaStream_t stream);
+    bool tiles_fit(const std::vector<Seg>& segs) const;
+    static bool pages_are_run(const Seg& s) {
+        for (uint32_t k = 1; k < s.n_pages; ++k)
+            if (s.pages[k] != s.pages[0] + k) return false;
+        return true;
+    }
     // the call's stream in the dependency tracker (creating its events), and
     // the work counter its launches use
     t2i_status stream_slot(cudaStream_t s, int* si) {
@@ -260,6 +271,7 @@ class Store {
     static constexpr size_t kCompactFirstBatch = T2I_TUNE_COMPACT_FIRST;  // moves in the first launch
     static_assert(kMovesPerLaunch * (sizeof(SegDesc) + sizeof(uint32_t)) <= size_t(kBlobLarge), "moves per launch");
     std::vector<SegDesc> sd_;
+    std::vector<TileSeg> ts_;
     std::vector<uint32_t> lp_;
     alignas(16) unsigned char param_buf_[sizeof(LaunchParams<kBlobLarge>)];
 };

@@ -1,0 +1,65 @@
+"""Tiled launches (marked gpu) at the sizes where a tile can go wrong: objects
+that end around a 16 KiB tile, pages of one tile and larger, pages smaller
+than a tile (only runs of them are tiled), scattered and consecutive pages,
+with and without the cast; put, get, compaction and pull. Every byte against
+the input, the casts against the oracle's round-to-nearest-even."""
+import numpy as np
+import pytest
+import torch
+
+from oracle.cast import f32_bits_to_bf16_bits
+from paper_2607_26566_gb300 import Store, get_descs, put_descs
+
+pytestmark = pytest.mark.gpu
+DEV = torch.device("cuda", 0)
+TILE = 16384
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built(lib):
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    yield
+
+
+def scatter(st, n_pages, P, seed):
+    """Free pages in a shuffled order."""
+    s, ids = st.put_batch(put_descs(np.zeros(n_pages, np.uint64), nbytes=np.full(n_pages, P)))
+    assert s == 0
+    assert st.free(np.random.default_rng(seed).permutation(ids)) == 0
+
+
+@pytest.mark.parametrize("big", [24 << 20, 256 << 10])   # a launch of many tiles, and a small one
+@pytest.mark.parametrize("P,policy", [(16384, 0), (65536, 0), (2 << 20, 0), (4096, 1)])
+def test_objects_that_end_around_a_tile(P, policy, big):
+    rng = np.random.default_rng(P + policy)
+    sizes = [big + 4] + [k * TILE + d for k in (1, 3) for d in (-16, -4, 0, 4, 16, 36)] + [4, 2 * P, 2 * P + 12]
+    casts = [0] + [k % 2 for k in range(len(sizes) - 1)]
+    datas = [rng.integers(0, 256, n, dtype=np.uint8) for n in sizes]
+    n_pages = 2 * (sum(-(-n // P) for n in sizes) + 8)
+    st = Store(torch.zeros(n_pages * P, dtype=torch.uint8, device=DEV), P, alloc_policy=policy)
+    if policy == 0:
+        scatter(st, n_pages, P, 3)
+    srcs = [torch.from_numpy(d).to(DEV) for d in datas]
+    s, dead = st.put_batch(put_descs([0], nbytes=[(n_pages // 2) * P]))
+    s, ids = st.put_batch(put_descs(srcs))
+    assert s == 0, st.last_error()
+    want = [f32_bits_to_bf16_bits(d.view(np.uint32)).view(np.uint8) if c else d for d, c in zip(datas, casts)]
+
+    def check(store, which):
+        outs = [torch.full((w.size + 32,), 0xCD, dtype=torch.uint8, device=DEV) for w in want]
+        assert store.get_batch(get_descs(which, outs, dst_bytes=[w.size for w in want], cast=casts))[0] == 0
+        torch.cuda.synchronize()
+        for o, w, n in zip(outs, want, sizes):
+            h = o.cpu().numpy()
+            assert np.array_equal(h[:w.size], w), n
+            assert (h[w.size:] == 0xCD).all(), n
+
+    check(st, ids)
+    cons = Store(torch.zeros(n_pages * P, dtype=torch.uint8, device=DEV), P)
+    s, pulled, _ = cons.pull(st, ids)
+    assert s == 0
+    check(cons, pulled)
+    assert st.free(dead) == 0
+    s, moved = st.compact((n_pages // 2) * P)
+    assert s == 0 and moved > 0
+    check(st, ids)
