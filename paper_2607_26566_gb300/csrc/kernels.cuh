@@ -199,11 +199,26 @@ constexpr int kTileVec = T2I_TUNE_TILE_VEC;
 constexpr uint32_t kTileBytes = kTileThreads * kTileVec * 16;  // 16 KiB
 constexpr uint32_t kTileShift = kTileBytes == 8192 ? 13 : kTileBytes == 16384 ? 14 : kTileBytes == 32768 ? 15 : 16;
 static_assert(kTileBytes == 1u << kTileShift, "tile size");
-// Aligned launches of at least this many bytes run as tiles. Below it the
-// launch is bound by its latency, and the other kernels' 16 KiB shares are
-// the same size: eight B=1 requests (11.5 MB a call) took 89.3 us a pass in
-// those kernels and 69 in tiles, a 16 MiB get the same in both.
+// Aligned launches of at least this many bytes run as CTA tiles, others as
+// warp tiles. The line is broad: put + get of B=4 requests (45 MB a call) took
+// 93.9 us a pass in CTA tiles and 95.3 in warp tiles, of B=1 requests (11.5
+// MB) 69 in both, a 40 MB adapter get 12.2 and 12.0. Below it the launch is
+// bound by its latency, and a warp starts sooner than 512 threads.
 constexpr uint64_t kTileMinBytes = T2I_TUNE_TILE_MIN_BYTES;
+
+// Warp tiles (see warp_tile): 4 KiB each, one warp each, any alignment. CTAs
+// of 2, 4 or 8 warps ran alike (within 2%) on small and ragged batches.
+#ifndef T2I_TUNE_WARP_THREADS
+#define T2I_TUNE_WARP_THREADS 128
+#endif
+#ifndef T2I_TUNE_WARP_BLOCKS
+#define T2I_TUNE_WARP_BLOCKS 8
+#endif
+constexpr int kWarpThreads = T2I_TUNE_WARP_THREADS;
+constexpr int kWarpVec = 8;  // 16-byte source vectors per lane
+constexpr uint32_t kWarpTileShift = 12;
+constexpr uint32_t kWarpTileBytes = 1u << kWarpTileShift;
+static_assert(kWarpTileBytes == 32 * kWarpVec * 16, "one round of a warp's loads per tile");
 
 struct TileSeg {
     uint64_t user;
@@ -221,8 +236,8 @@ struct TileHeader {
     uint64_t pool;
     uint32_t n_seg;
     uint32_t page_shift;
-    uint32_t pages_offset;  // byte offset of the uint32 page array in blob
-    uint32_t flags;         // kPrefetchSources, or 0
+    uint32_t n_tiles;
+    uint32_t flags;  // kPrefetchSources, or 0
 };
 static_assert(sizeof(TileHeader) == 24, "TileHeader layout");
 
@@ -889,6 +904,19 @@ __device__ __forceinline__ void run_range(const LaunchParams<BLOB>& p, uint64_t 
     }
 }
 
+// The last segment that starts at or before this tile.
+__device__ __forceinline__ uint32_t find_tile(const TileSeg* segs, uint32_t n_seg, uint32_t tile) {
+    uint32_t lo = 0, hi = n_seg - 1;
+    while (lo < hi) {
+        const uint32_t mid = (lo + hi + 1) >> 1;
+        if (segs[mid].tile0 <= tile)
+            lo = mid;
+        else
+            hi = mid - 1;
+    }
+    return lo;
+}
+
 // ------------------------------------------------------------- tiled launches
 // One CTA per tile: the 16 KiB (or the rest) of one segment at a multiple of
 // 16 KiB, in one page or one run of pages, both sides 16-byte aligned. Bound
@@ -905,22 +933,14 @@ template <Mode M, int BLOB>
 __device__ __forceinline__ void tile_copy(const TileParams<BLOB>& p) {
     constexpr bool kToUser = M == Mode::Get;
     const TileSeg* segs = reinterpret_cast<const TileSeg*>(p.blob);
-    uint32_t lo = 0, hi = p.h.n_seg - 1;
-    while (lo < hi) {  // the last segment that starts at or before this tile
-        const uint32_t mid = (lo + hi + 1) >> 1;
-        if (segs[mid].tile0 <= blockIdx.x)
-            lo = mid;
-        else
-            hi = mid - 1;
-    }
+    const uint32_t lo = find_tile(segs, p.h.n_seg, blockIdx.x);
     const uint32_t off = (blockIdx.x - segs[lo].tile0) << kTileShift;
     const uint32_t len = umin(kTileBytes, segs[lo].nbytes - off);
     const uint32_t flags = segs[lo].flags;
     const bool cast = kToUser && (flags & kTileCast);
     uint32_t page = segs[lo].page, in_page = off;
     if (!(flags & kTileOnePage)) {
-        const uint32_t* pages = reinterpret_cast<const uint32_t*>(p.blob + p.h.pages_offset);
-        page = pages[page + (off >> p.h.page_shift)];
+        page = reinterpret_cast<const uint32_t*>(segs + p.h.n_seg)[page + (off >> p.h.page_shift)];
         in_page = off & ((1u << p.h.page_shift) - 1);
     }
     unsigned char* pa = reinterpret_cast<unsigned char*>(p.h.pool) + (uint64_t(page) << p.h.page_shift) + in_page;
@@ -934,6 +954,207 @@ __device__ __forceinline__ void tile_copy(const TileParams<BLOB>& p) {
         tile_cast(dst, src, len);
     else
         tile_copy_bytes(dst, src, len);
+}
+
+// ---------------------------------------------------------------- warp tiles
+// Bytes [n, n + 16) of lo|hi, n in 0..15.
+__device__ __forceinline__ uint4 bytes_from(uint4 lo, uint4 hi, uint32_t n) {
+    const bool by8 = n & 8u, by4 = n & 4u;
+    const uint32_t a0 = by8 ? lo.z : lo.x, a1 = by8 ? lo.w : lo.y, a2 = by8 ? hi.x : lo.z, a3 = by8 ? hi.y : lo.w,
+                   a4 = by8 ? hi.z : hi.x, a5 = by8 ? hi.w : hi.y;
+    const uint32_t b0 = by4 ? a1 : a0, b1 = by4 ? a2 : a1, b2 = by4 ? a3 : a2, b3 = by4 ? a4 : a3, b4 = by4 ? a5 : a4;
+    const uint32_t r = 8u * (n & 3u);
+    return make_uint4(__funnelshift_r(b0, b1, r), __funnelshift_r(b1, b2, r), __funnelshift_r(b2, b3, r),
+                      __funnelshift_r(b3, b4, r));
+}
+
+__device__ __forceinline__ uint4 shfl4(uint4 v, uint32_t from) {
+    return make_uint4(__shfl_sync(0xFFFFFFFFu, v.x, from), __shfl_sync(0xFFFFFFFFu, v.y, from),
+                      __shfl_sync(0xFFFFFFFFu, v.z, from), __shfl_sync(0xFFFFFFFFu, v.w, from));
+}
+
+// Stores output vectors d[first .. nv): d[k] = bytes [n, n + 16) of w[k]|w[k + 1].
+// Lane l holds w[32 j + l] in r[j], lane 31 also w[32 V] in last.
+template <int V>
+__device__ __forceinline__ void store_shifted(uint4* d, const uint4 (&r)[V], uint4 last, uint32_t n, uint32_t first,
+                                              uint32_t nv) {
+    const uint32_t lane = threadIdx.x & 31u;
+#pragma unroll
+    for (int j = 0; j < V; ++j) {
+        // the next vector: lane + 1's, or for lane 31 lane 0's of the next 32
+        uint4 next = shfl4(j + 1 < V && lane == 0 ? r[j + 1 < V ? j + 1 : j] : r[j], (lane + 1) & 31u);
+        if (j + 1 == V && lane == 31) next = last;
+        const uint32_t k = j * 32 + lane;
+        if (k >= first && k < nv) st_stream(d + k, bytes_from(r[j], next, n));
+    }
+}
+
+// One warp per tile: 4 KiB of one segment's source, at any alignment of the
+// user's address, pages of any size. No shared memory, no barrier: a warp
+// finds its tile, asks L2 for its source lines and then waits for the
+// previous grid; every global access but a segment's first and last bytes
+// is one aligned 16-byte vector. Where the two sides are misaligned to each
+// other, each output vector is cut out of two source vectors, the second
+// one taken from the next lane (a shuffle). Tiles are cut at 16-byte
+// boundaries of the side that is written, so that only a segment's first
+// and last vectors are partial.
+// Bound by latency in small launches: a warp holds 4 KiB of one segment, so
+// that many small segments run side by side instead of one after another in
+// a CTA's share, and a call with any mix of alignments is one launch instead
+// of two. Bound by HBM in large ones, which come here for their alignment or
+// their small pages. Before (CTAs walking shares, pieces realigned in shared
+// memory) and after: 646 tensors of 256 B to 36 KiB got in 30.8 -> 25.3 us, 40
+// ragged objects put and got in 18.5 -> 15.9; 1 GiB puts from unaligned
+// sources 7.13 -> 7.21 TB/s, gets into unaligned destinations 7.08 -> 7.13,
+// casts into 2-byte aligned ones 6.92 -> 7.18; 64 MiB in scattered 8 KiB pages
+// put 4.97 -> 7.25, got 4.81 -> 6.50, cast 3.24 -> 6.53.
+template <Mode M, int BLOB>
+__device__ __forceinline__ void warp_tile(const TileParams<BLOB>& p) {
+    constexpr bool kToUser = M == Mode::Get;
+    const uint32_t lane = threadIdx.x & 31u;
+    const uint32_t tile = blockIdx.x * (kWarpThreads / 32) + (threadIdx.x >> 5);
+    if (tile >= p.h.n_tiles) {
+        pdl_wait_then_release();
+        return;
+    }
+    const TileSeg* segs = reinterpret_cast<const TileSeg*>(p.blob);
+    const TileSeg& s = segs[find_tile(segs, p.h.n_seg, tile)];
+    const uint32_t* pages = reinterpret_cast<const uint32_t*>(segs + p.h.n_seg);
+    unsigned char* pool = reinterpret_cast<unsigned char*>(p.h.pool);
+    unsigned char* user = reinterpret_cast<unsigned char*>(s.user);
+    const uint32_t nbytes = s.nbytes, flags = s.flags, page = s.page, pshift = p.h.page_shift;
+    const uint32_t at = (tile - s.tile0) << kWarpTileShift;  // source bytes before this tile (less the phase)
+    const uint32_t phase = uint32_t(s.user) & 15u;           // of the user's side; pages are 16-byte aligned
+    // pool address of byte o of the segment
+    auto paged = [&](uint32_t o) -> unsigned char* {
+        if (flags & kTileOnePage) return pool + (uint64_t(page) << pshift) + o;
+        return pool + (uint64_t(pages[page + (o >> pshift)]) << pshift) + (o & ((1u << pshift) - 1));
+    };
+    // the same for bytes of this tile, whose page (or run) is looked up once
+    const bool one_page = (flags & kTileOnePage) || pshift >= kWarpTileShift;
+    unsigned char* const base = one_page && at < nbytes ? paged(at) : pool;
+    auto in_tile = [&](uint32_t o) -> unsigned char* { return one_page ? base + (o - at) : paged(o); };
+
+    if (kPrefetch && (p.h.flags & kPrefetchSources) && at + lane * 128u < nbytes)
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(kToUser ? in_tile(at + lane * 128u) : user + at + lane * 128u));
+    pdl_wait_then_release();
+
+    if (kToUser && (flags & kTileCast)) {
+        // fp32 -> bf16: blocks of 8 floats (32 bytes) make one output vector.
+        // With q counting output bytes from the 16-byte boundary at or before
+        // `user`, the tile is q in [at / 2, at / 2 + 2048) and its vector k
+        // holds the last phase bytes of block at / 32 + k - 1 and the first of
+        // block at / 32 + k.
+        constexpr int kBlocks = kWarpVec / 2;
+        const uint32_t nq = umin((nbytes >> 1) + phase - (at >> 1), kWarpTileBytes / 2);
+        const uint32_t nv = nq >> 4;
+        uint16_t* d16 = reinterpret_cast<uint16_t*>(user - phase + (at >> 1));
+        const uint32_t back = phase ? 32u : 0u;  // w[0] is the block before the tile's
+        const uint32_t need = phase ? nv + 1 : nv;
+        const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+        auto load = [&](uint32_t k, uint4* a, uint4* b) {  // the two vectors of w[k]; those without a source byte are zero
+            const uint32_t o = at + 32u * k - back;
+            *a = *b = zero;
+            if (k >= need || int32_t(o) < 0 || o >= nbytes) return;
+            const unsigned char* src = o < at ? paged(o) : in_tile(o);
+            *a = ld_stream(reinterpret_cast<const uint4*>(src));
+            if (o + 16u < nbytes) *b = ld_stream(reinterpret_cast<const uint4*>(src) + 1);
+        };
+        auto bf16 = [](const uint4& a, const uint4& b) {
+            return make_uint4(pack_bf16x2(a.x, a.y), pack_bf16x2(a.z, a.w), pack_bf16x2(b.x, b.y), pack_bf16x2(b.z, b.w));
+        };
+        uint4 a[kBlocks], b[kBlocks], la = zero, lb = zero;
+#pragma unroll
+        for (int j = 0; j < kBlocks; ++j) load(j * 32 + lane, &a[j], &b[j]);
+        if (phase && lane == 31) load(kBlocks * 32, &la, &lb);
+        // the elements before the first whole vector and after the last one
+        const bool head = phase && at == 0;
+        const uint32_t n_head = head ? umin((16u - phase) >> 1, nbytes >> 2) : 0u;
+        const uint32_t n_tail = head && nv == 0 ? 0u : (nq & 15u) >> 1;
+        const uint32_t e_head = phase >> 1, e_tail = nv << 3;
+        uint16_t x_head = 0, x_tail = 0;
+        if (lane < n_head) x_head = (uint16_t)bf16_rne_bits(*reinterpret_cast<const uint32_t*>(paged(4u * lane)));
+        if (lane < n_tail)
+            x_tail = (uint16_t)bf16_rne_bits(*reinterpret_cast<const uint32_t*>(paged(at + 4u * (e_tail + lane - e_head))));
+        uint4* d = reinterpret_cast<uint4*>(d16);
+        uint4 r[kBlocks];
+#pragma unroll
+        for (int j = 0; j < kBlocks; ++j) r[j] = bf16(a[j], b[j]);
+        if (phase) {
+            store_shifted<kBlocks>(d, r, bf16(la, lb), 16u - phase, head ? 1u : 0u, nv);
+        } else {
+#pragma unroll
+            for (int j = 0; j < kBlocks; ++j)
+                if (j * 32 + lane < nv) st_stream(d + j * 32 + lane, r[j]);
+        }
+        if (lane < n_head) d16[e_head + lane] = x_head;
+        if (lane < n_tail) d16[e_tail + lane] = x_tail;
+        return;
+    }
+
+    // A copy. With q counting bytes from the 16-byte boundary at or before
+    // the first byte written (q = byte + skip), the tile is q in
+    // [at, at + 4096). Output vector k is bytes [n, n + 16) of w[k]|w[k + 1]:
+    // get: w[k] = the object's vector at / 16 + k - 1, n = 16 - phase;
+    // put: w[k] = the user's aligned vector at / 16 + k, n = phase.
+    const uint32_t skip = kToUser ? phase : 0u;
+    const uint32_t nq = umin(nbytes + skip - at, kWarpTileBytes);
+    const uint32_t nv = nq >> 4;
+    unsigned char* const out = kToUser ? user - phase + at : nullptr;
+    const unsigned char* const in = kToUser ? nullptr : user - phase + at;
+    auto w = [&](uint32_t k) -> uint4 {
+        const unsigned char* a;
+        if (kToUser) {
+            const uint32_t o = at + 16u * k - (phase ? 16u : 0u);
+            if (int32_t(o) < 0 || o >= nbytes) return make_uint4(0u, 0u, 0u, 0u);
+            a = o < at ? paged(o) : in_tile(o);
+        } else {
+            a = in + 16u * k;
+        }
+        return ld_stream(reinterpret_cast<const uint4*>(a));
+    };
+    const uint32_t need = phase ? nv + 1 : nv;
+    uint4 r[kWarpVec], last = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+    for (int j = 0; j < kWarpVec; ++j) r[j] = (nv && j * 32 + lane < need) ? w(j * 32 + lane) : last;
+    if (phase && lane == 31 && need > kWarpVec * 32) last = w(kWarpVec * 32);
+    const bool head = skip && at == 0;
+    const uint32_t n_head = head ? umin(16u - phase, nbytes) : 0u;
+    const uint32_t n_tail = head && nv == 0 ? 0u : nq & 15u;
+    const uint32_t o_tail = at + (nv << 4) - skip;  // first byte after the last whole vector
+    unsigned char x_head = 0, x_tail = 0;
+    if (kToUser && lane < n_head) x_head = *paged(lane);
+    if (lane < n_tail) x_tail = kToUser ? *paged(o_tail + lane) : user[o_tail + lane];
+    const uint32_t first = head ? 1u : 0u, n = kToUser ? 16u - phase : phase;
+    if (kToUser || one_page) {
+        uint4* d = reinterpret_cast<uint4*>(kToUser ? out : base);
+        if (phase) {
+            store_shifted<kWarpVec>(d, r, last, n, first, nv);
+        } else {
+#pragma unroll
+            for (int j = 0; j < kWarpVec; ++j)
+                if (j * 32 + lane < nv) st_stream(d + j * 32 + lane, r[j]);
+        }
+    } else {  // pages smaller than a tile: each vector finds its own
+#pragma unroll
+        for (int j = 0; j < kWarpVec; ++j) {
+            uint4 v = r[j];
+            if (phase) {
+                uint4 next = shfl4(j + 1 < kWarpVec && lane == 0 ? r[j + 1 < kWarpVec ? j + 1 : j] : r[j], (lane + 1) & 31u);
+                if (j + 1 == kWarpVec && lane == 31) next = last;
+                v = bytes_from(v, next, n);
+            }
+            const uint32_t k = j * 32 + lane;
+            if (k < nv) st_stream(reinterpret_cast<uint4*>(paged(at + 16u * k)), v);
+        }
+    }
+    if (kToUser && lane < n_head) user[lane] = x_head;
+    if (lane < n_tail) {
+        if (kToUser)
+            user[o_tail + lane] = x_tail;
+        else
+            *paged(o_tail + lane) = x_tail;
+    }
 }
 
 // Named entry points (one per operation, so that profiles name them).
@@ -959,6 +1180,16 @@ __global__ void __launch_bounds__(kThreads, GENERAL ? kMinBlocksGeneral : kMinBl
     prefetch_share<Mode::GetCopy, BLOB>(p);
     pdl_wait_then_release();
     run_share<Mode::GetCopy, GENERAL, BLOB>(p);
+}
+template <int BLOB>
+__global__ void __launch_bounds__(kWarpThreads, T2I_TUNE_WARP_BLOCKS)
+    put_warp_kernel(const __grid_constant__ TileParams<BLOB> p) {
+    warp_tile<Mode::Put, BLOB>(p);
+}
+template <int BLOB>
+__global__ void __launch_bounds__(kWarpThreads, T2I_TUNE_WARP_BLOCKS)
+    get_warp_kernel(const __grid_constant__ TileParams<BLOB> p) {
+    warp_tile<Mode::Get, BLOB>(p);
 }
 template <int BLOB>
 __global__ void __launch_bounds__(kTileThreads, T2I_TUNE_TILE_BLOCKS)

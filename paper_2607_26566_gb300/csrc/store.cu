@@ -115,56 +115,12 @@ class Store {
         handle_.owned = false;
         handle_.mu = &mu;
         page_shift_ = log2_exact(cfg.page_bytes);
+        deps_.resize_pages(ctl_.total_pages());
     }
     ~Store() {
         DeviceGuard g(device_);
         deps_.synchronize_all();
         deps_.release();
-        if (work_) cudaFree(work_);
-    }
-
-    t2i_status init(std::string* err) {
-        DeviceGuard g(device_);
-        int sms = 0;
-        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device_) != cudaSuccess || sms <= 0) {
-            *err = "cannot query the device";
-            return T2I_ERR_CUDA;
-        }
-        // resident CTAs on the device (SMs x CTAs per SM), per kernel
-        const void* fns[4][2] = {
-            {reinterpret_cast<const void*>(scatter_put_kernel<kBlobLarge, false>),
-             reinterpret_cast<const void*>(scatter_put_kernel<kBlobLarge, true>)},
-            {reinterpret_cast<const void*>(gather_get_kernel<kBlobLarge, false>),
-             reinterpret_cast<const void*>(gather_get_kernel<kBlobLarge, true>)},
-            {reinterpret_cast<const void*>(compact_move_kernel<kBlobLarge>),
-             reinterpret_cast<const void*>(compact_move_kernel<kBlobLarge>)},
-            {reinterpret_cast<const void*>(gather_copy_kernel<kBlobLarge, false>),
-             reinterpret_cast<const void*>(gather_copy_kernel<kBlobLarge, true>)}};
-        for (int m = 0; m < 4; ++m)
-            for (int a = 0; a < 2; ++a) {
-                int occ = 0;
-                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fns[m][a], kThreads, 0);
-                max_ctas_[m][a] = sms * (occ > 0 ? occ : 1);
-            }
-        // one chunk counter per stream (the first kWorkStreams streams of
-        // the store; later ones use equal static shares), zeroed once
-        if (cudaMalloc(&work_, kWorkStreams * sizeof(WorkCounter)) != cudaSuccess) {
-            work_ = nullptr;
-            *err = "cannot allocate the work counters";
-            return T2I_ERR_CUDA;
-        }
-        // cleared on a private non-blocking stream: waits for nothing else
-        cudaStream_t zs = nullptr;
-        bool zeroed = cudaStreamCreateWithFlags(&zs, cudaStreamNonBlocking) == cudaSuccess &&
-                      cudaMemsetAsync(work_, 0, kWorkStreams * sizeof(WorkCounter), zs) == cudaSuccess &&
-                      cudaStreamSynchronize(zs) == cudaSuccess;
-        if (zs) cudaStreamDestroy(zs);
-        if (!zeroed) {
-            *err = "cannot clear the work counters";
-            return T2I_ERR_CUDA;
-        }
-        deps_.resize_pages(ctl_.total_pages());
-        return T2I_OK;
     }
 
     std::mutex mu;
@@ -207,32 +163,23 @@ class Store {
     };
     template <Mode M>
     t2i_status launch_segments(const std::vector<Seg>& segs, cudaStream_t stream);
-    template <Mode M, bool GENERAL>
-    t2i_status launch_group(const std::vector<Seg>& segs, cudaStream_t stream);
-    template <Mode M, bool GENERAL, int BLOB>
-    t2i_status launch_one(const std::vector<SegDesc>& sd, const std::vector<uint32_t>& pages, uint32_t n_granules,
-                          cudaStream_t stream);
     t2i_status launch_kernel(const void* fn, unsigned grid, unsigned threads, cudaStream_t stream);
-    template <Mode M>
+    template <Mode M, bool WARP>
     t2i_status launch_tiles(const std::vector<Seg>& segs, cudaStream_t stream);
-    template <Mode M, int BLOB>
-    t2i_status launch_tiles_one(uint32_t n_tiles, cudaStream_t stream);
-    bool tiles_fit(const std::vector<Seg>& segs) const;
+    template <Mode M, bool WARP, int BLOB>
+    t2i_status launch_tiles_one(uint32_t n_seg, uint32_t n_tiles, cudaStream_t stream);
     static bool pages_are_run(const Seg& s) {
         for (uint32_t k = 1; k < s.n_pages; ++k)
             if (s.pages[k] != s.pages[0] + k) return false;
         return true;
     }
-    // the call's stream in the dependency tracker (creating its events), and
-    // the work counter its launches use
+    // the call's stream in the dependency tracker (creating its events)
     t2i_status stream_slot(cudaStream_t s, int* si) {
         *si = deps_.stream_index(s);
         if (*si < 0) {
             err_ = "cannot create the events for a new stream";
             return T2I_ERR_CUDA;
         }
-        cur_work_ = *si < int(kWorkStreams) ? reinterpret_cast<uint64_t>(work_) + uint64_t(*si) * sizeof(WorkCounter)
-                                             : 0;
         return T2I_OK;
     }
     t2i_status cuda_fail(const char* what, cudaError_t e) {
@@ -246,16 +193,9 @@ class Store {
     Control ctl_;
     t2i_ctl handle_{};
     uint32_t page_shift_ = 0;
-    int max_ctas_[4][2] = {{1, 1}, {1, 1}, {1, 1}, {1, 1}};  // [mode][any alignment]: resident CTAs on the device
     uint32_t fail_countdown_ = 0;  // > 0: that many launches from now, report a failure (testing)
-    // Work counters, one per stream index: launches on one stream run one
-    // after another (each waits for the previous grid before touching its
-    // counter), launches on different streams use different counters.
-    static constexpr uint32_t kWorkStreams = 64;
-    WorkCounter* work_ = nullptr;
-    uint64_t cur_work_ = 0;  // the current call's counter (0: static shares)
-    // LaunchHeader::flags of the current call's launches with static
-    // shares: kPrefetchSources unless a put reads host or managed memory
+    // TileHeader::flags of the current call's launches: kPrefetchSources
+    // unless a put reads host or managed memory
     uint32_t launch_flags_ = kPrefetchSources;
     std::vector<Seg> aligned_, general_;
     StreamDeps deps_;
@@ -263,17 +203,15 @@ class Store {
     std::vector<const Object*> objs_;
     std::vector<Seg> segs_;
     std::vector<t2i_move> batch_;  // the moves of one compaction launch
-    // moves per compaction launch: one 24-byte descriptor and one page each
+    // moves per compaction launch: one 24-byte descriptor each
     static constexpr size_t kMovesPerLaunch = 1024;
 #ifndef T2I_TUNE_COMPACT_FIRST
 #define T2I_TUNE_COMPACT_FIRST 64
 #endif
     static constexpr size_t kCompactFirstBatch = T2I_TUNE_COMPACT_FIRST;  // moves in the first launch
-    static_assert(kMovesPerLaunch * (sizeof(SegDesc) + sizeof(uint32_t)) <= size_t(kBlobLarge), "moves per launch");
-    std::vector<SegDesc> sd_;
-    std::vector<TileSeg> ts_;
+    static_assert(kMovesPerLaunch * sizeof(TileSeg) <= size_t(kBlobLarge), "moves per launch");
     std::vector<uint32_t> lp_;
-    alignas(16) unsigned char param_buf_[sizeof(LaunchParams<kBlobLarge>)];
+    alignas(16) unsigned char param_buf_[sizeof(TileParams<kBlobLarge>)];
 };
 
 t2i_status Store::check_user(const void* p, uint64_t n, bool want_write, bool is_host_flag, uint64_t* dev_addr,
@@ -898,13 +836,6 @@ t2i_status t2i_store_create(void* pool_dev, const t2i_store_config* cfg, int dev
     } catch (const std::exception& e) {
         t2i::set_thread_error(std::string("t2i_store_create: host error: ") + e.what());
         return T2I_ERR_INVALID;
-    }
-    std::string err;
-    t2i_status st = s->init(&err);
-    if (st != T2I_OK) {
-        delete s;
-        t2i::set_thread_error("t2i_store_create: " + err);
-        return st;
     }
     *out = new t2i_store{s};
     return T2I_OK;

@@ -63,3 +63,35 @@ def test_objects_that_end_around_a_tile(P, policy, big):
     s, moved = st.compact((n_pages // 2) * P)
     assert s == 0 and moved > 0
     check(st, ids)
+
+
+@pytest.mark.parametrize("P", [256, 2048, 4096, 65536])
+@pytest.mark.parametrize("mis", [0, 1, 8, 14, 15])
+def test_warp_tiles_at_their_edges(P, mis):
+    """Small launches (warp tiles of 4 KiB): objects that end around a 16-byte
+    vector and around a tile, sources and destinations `mis` bytes past a
+    16-byte boundary, scattered pages smaller and larger than a tile, casts
+    and copies in one call; the bytes around every destination stay."""
+    rng = np.random.default_rng(P + mis)
+    sizes = [k + d for k in (16, 4096, 8192, 40960) for d in (-15, -4, -1, 0, 1, 4, 15)] + [4, 8, 300 * P // 256]
+    casts = [int(n % 4 == 0 and mis % 2 == 0) for n in sizes]
+    datas = [rng.integers(0, 256, n, dtype=np.uint8) for n in sizes]
+    n_pages = sum(-(-n // P) for n in sizes) + 3
+    st = Store(torch.zeros(n_pages * P, dtype=torch.uint8, device=DEV), P)
+    scatter(st, n_pages, P, 5)
+    bufs = [torch.zeros(mis + n, dtype=torch.uint8, device=DEV) for n in sizes]
+    for b, d in zip(bufs, datas):
+        b[mis:] = torch.from_numpy(d).to(DEV)
+    s, ids = st.put_batch(put_descs([b.data_ptr() + mis for b in bufs], nbytes=sizes))
+    assert s == 0, st.last_error()
+    assert st.stats()["launches"] == 1  # any mix of alignments is one launch
+    for cast in (casts, [0] * len(sizes)):
+        want = [f32_bits_to_bf16_bits(d.view(np.uint32)).view(np.uint8) if c else d for d, c in zip(datas, cast)]
+        outs = [torch.full((mis + w.size + 32,), 0xCD, dtype=torch.uint8, device=DEV) for w in want]
+        assert st.get_batch(get_descs(ids, [o.data_ptr() + mis for o in outs], dst_bytes=[w.size for w in want],
+                                      cast=cast))[0] == 0
+        torch.cuda.synchronize()
+        for o, w, n in zip(outs, want, sizes):
+            h = o.cpu().numpy()
+            assert np.array_equal(h[mis:mis + w.size], w), n
+            assert (h[:mis] == 0xCD).all() and (h[mis + w.size:] == 0xCD).all(), n
