@@ -335,9 +335,7 @@ t2i_status t2i_inject_launch_failure(t2i_store* store, uint32_t countdown);
 /* Copies one object's pages out of a pool into a contiguous device buffer,
  * with the same bytes and the same optional fp32 -> bf16 RNE cast as a
  * one-item t2i_get_batch, but with no store and without allocating any
- * memory. Its launches are those of a store's chunked get: the cast-capable
- * gather kernel for a 16-byte aligned destination or a cast, the copy-only
- * gather kernel for any other destination.
+ * memory. Its launches are those of such a get.
  *
  * Who needs it: a caller that must not allocate device memory while it
  * moves data. In a serving process the free HBM is often reserved up front
@@ -345,26 +343,21 @@ t2i_status t2i_inject_launch_failure(t2i_store* store, uint32_t countdown);
  * cudaMalloc there fails, and a cudaFree waits for the whole device. Code
  * that holds a pool and its page lists but no t2i_store uses it too.
  *
- * Scratch: the CTAs of a launch take their chunks from counters kept in a
- * static 2 KiB device array of the library (64 counters of 32 bytes: one
- * per launch of a call). Every GPU that loads the library holds the array
- * until the process exits. A call first zeroes the counters it will use
- * (cudaMemsetAsync on cuda_stream), because every call shares the array and
- * it keeps whatever the last call left. Calls that overlap on the GPU (on
- * other streams or from other threads) race on the counters and can skip or
- * repeat chunks: order such calls on one stream. The first call on a device
- * sets up that device: it looks up the array's device address
- * (cudaGetSymbolAddress) and the gather kernels' occupancy. Make that first
- * call before any stream capture. No call allocates: no cudaMalloc, no
- * cudaFree, no library routine that allocates.
+ * It needs no scratch memory: what a launch copies stands in its parameters,
+ * so calls may overlap on any streams and threads. The first call on a device
+ * loads the gather kernels there (the driver keeps their code in device
+ * memory); make that call before any stream capture. No other call allocates
+ * device memory: no cudaMalloc, no cudaFree, no library routine that
+ * allocates.
  *
  * pool_dev, pool_bytes: the pool, device memory of `device`; pool_bytes is a
  *   positive multiple of page_bytes, a power of two in [256 B, 1 GiB].
  * pages, n_pages: the object's page list in byte order (a host array of
  *   page indices into the pool, e.g. from t2i_ctl_object), read during the
- *   call. n_pages = ceil(nbytes / page_bytes), at most 64 launches of
- *   min(7,930, 64 GiB / page_bytes) pages, one scratch counter each: 507,520
- *   pages for pages up to 8 MiB. Larger objects are INVALID.
+ *   call. n_pages = ceil(nbytes / page_bytes), at most 64 times
+ *   min(7,930, 64 GiB / page_bytes) pages (7,930 scattered pages fit one
+ *   launch's parameters): 507,520 pages for pages up to 8 MiB. Larger objects
+ *   are INVALID.
  * nbytes: the object's size. dst_dev, dst_bytes: the destination, device
  *   memory of `device` that does not overlap the pool. cast = 1 writes bf16
  *   (nbytes % 4 == 0, even dst_dev, dst_bytes >= nbytes / 2); cast = 0

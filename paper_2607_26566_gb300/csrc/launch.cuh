@@ -1,61 +1,109 @@
-// Launch packing of the store's kernels (part of store.cu; included after
-// the Store class). A batch's segments are packed into as few launches as
-// their descriptors allow (each launch carries up to ~31 KiB of descriptors
-// and page numbers in its parameters), as CTA tiles or as warp tiles, and
-// launched with programmatic dependent launch. Together with kernels.cuh
-// this decides what a launch does, so profiles are keyed to a hash of both
-// files. Included by store.cu inside namespace t2i.
+// Launch packing of the store's kernels (part of store.cu). A batch's segments
+// are packed into as few launches as their descriptors allow (each launch
+// carries up to ~31 KiB of descriptors and page numbers in its parameters),
+// as CTA tiles or as warp tiles, and launched with programmatic dependent
+// launch. Together with kernels.cuh this decides what a launch does, so
+// profiles are keyed to a hash of both files. Included by store.cu inside
+// namespace t2i.
 #pragma once
 
-// One kernel launch of the parameters in param_buf_.
-inline t2i_status Store::launch_kernel(const void* fn, unsigned grid, unsigned threads, cudaStream_t stream) {
-    void* args[] = {param_buf_};
-    if (fail_countdown_ && --fail_countdown_ == 0) {
-        err_ = "kernel launch failed: injected failure (t2i_inject_launch_failure)";
+// One object (or page) of a batch, on its way to a launch.
+struct Seg {
+    uint64_t user;          // device-visible address of the user's side
+    uint64_t nbytes_flags;  // bytes in the pool, kCastFlag
+    const uint32_t* pages;
+    uint32_t n_pages;
+};
+constexpr uint64_t kCastFlag = uint64_t(1) << 63;
+constexpr uint64_t kSegBytesMask = ~kCastFlag;
+
+inline bool pages_are_run(const Seg& s) {
+    for (uint32_t k = 1; k < s.n_pages; ++k)
+        if (s.pages[k] != s.pages[0] + k) return false;
+    return true;
+}
+
+// The kernel of a mode, a kind of tile and a tier of parameters.
+template <Mode M, bool WARP, int BLOB>
+const void* tile_kernel() {
+    if constexpr (WARP)
+        return M == Mode::Get ? reinterpret_cast<const void*>(gather_get_warp_kernel<BLOB>)
+                              : reinterpret_cast<const void*>(scatter_put_warp_kernel<BLOB>);
+    else
+        return M == Mode::Put   ? reinterpret_cast<const void*>(scatter_put_kernel<BLOB>)
+               : M == Mode::Get ? reinterpret_cast<const void*>(gather_get_kernel<BLOB>)
+                                : reinterpret_cast<const void*>(compact_move_kernel<BLOB>);
+}
+
+// Packs and launches the segments of one pool.
+class TileLauncher {
+  public:
+    // launches (nullable) counts the kernels launched
+    TileLauncher(uint64_t pool, uint32_t page_shift, uint64_t* launches)
+        : pool_(pool), page_shift_(page_shift), launches_(launches) {}
+
+    // kPrefetchSources, or 0 when a source is (or may be) other than device memory
+    uint32_t flags = kPrefetchSources;
+    uint32_t fail_countdown = 0;  // > 0: that many launches from now, report a failure (testing)
+    std::string error;
+
+    template <Mode M>
+    t2i_status launch(const std::vector<Seg>& segs, cudaStream_t stream);
+
+  private:
+    template <Mode M, bool WARP>
+    t2i_status launch_tiles(const std::vector<Seg>& segs, cudaStream_t stream);
+    template <Mode M, bool WARP, int BLOB>
+    t2i_status launch_one(uint32_t n_seg, uint32_t n_tiles, cudaStream_t stream);
+
+    uint64_t pool_;
+    uint32_t page_shift_;
+    uint64_t* launches_;
+    std::vector<Seg> aligned_, general_;
+    std::vector<uint32_t> lp_;  // page lists of the launch being packed
+    alignas(16) unsigned char param_buf_[sizeof(TileParams<kBlobLarge>)];
+};
+
+// One launch of the n_seg descriptors in param_buf_ and the pages in lp_.
+template <Mode M, bool WARP, int BLOB>
+t2i_status TileLauncher::launch_one(uint32_t n_seg, uint32_t n_tiles, cudaStream_t stream) {
+    if (fail_countdown && --fail_countdown == 0) {
+        error = "kernel launch failed: injected failure (t2i_inject_launch_failure)";
         return T2I_ERR_CUDA;
     }
+    auto* p = reinterpret_cast<TileParams<BLOB>*>(param_buf_);
+    p->h.pool = pool_;
+    p->h.n_seg = n_seg;
+    p->h.page_shift = page_shift_;
+    p->h.n_tiles = n_tiles;
+    p->h.flags = flags;
+    std::memcpy(p->blob + n_seg * sizeof(TileSeg), lp_.data(), lp_.size() * sizeof(uint32_t));
+    constexpr uint32_t kPerCta = WARP ? kWarpThreads / 32 : 1;
+    void* args[] = {param_buf_};
     cudaLaunchConfig_t lc = {};
-    lc.gridDim = dim3(grid);
-    lc.blockDim = dim3(threads);
-    lc.dynamicSmemBytes = 0;
+    lc.gridDim = dim3((n_tiles + kPerCta - 1) / kPerCta);
+    lc.blockDim = dim3(WARP ? kWarpThreads : kTileThreads);
     lc.stream = stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     lc.attrs = attr;
     lc.numAttrs = 1;
-    cudaError_t e = cudaLaunchKernelExC(&lc, fn, args);
+    const cudaError_t e = cudaLaunchKernelExC(&lc, tile_kernel<M, WARP, BLOB>(), args);
     if (e != cudaSuccess) {
-        err_ = std::string("kernel launch failed: ") + cudaGetErrorString(e);
+        error = std::string("kernel launch failed: ") + cudaGetErrorString(e);
         return T2I_ERR_CUDA;
     }
-    ctl_.counters().launches++;
+    if (launches_) ++*launches_;
     return T2I_OK;
-}
-
-template <Mode M, bool WARP, int BLOB>
-t2i_status Store::launch_tiles_one(uint32_t n_seg, uint32_t n_tiles, cudaStream_t stream) {
-    auto* p = reinterpret_cast<TileParams<BLOB>*>(param_buf_);
-    p->h.pool = pool_;
-    p->h.n_seg = n_seg;
-    p->h.page_shift = page_shift_;
-    p->h.n_tiles = n_tiles;
-    p->h.flags = launch_flags_;
-    std::memcpy(p->blob + n_seg * sizeof(TileSeg), lp_.data(), lp_.size() * sizeof(uint32_t));
-    const void* fn = WARP ? (M == Mode::Get ? reinterpret_cast<const void*>(get_warp_kernel<BLOB>)
-                                            : reinterpret_cast<const void*>(put_warp_kernel<BLOB>))
-                          : (M == Mode::Put   ? reinterpret_cast<const void*>(put_tile_kernel<BLOB>)
-                             : M == Mode::Get ? reinterpret_cast<const void*>(get_tile_kernel<BLOB>)
-                                              : reinterpret_cast<const void*>(move_tile_kernel<BLOB>));
-    constexpr uint32_t kPerCta = WARP ? kWarpThreads / 32 : 1;
-    return launch_kernel(fn, (n_tiles + kPerCta - 1) / kPerCta, WARP ? kWarpThreads : kTileThreads, stream);
 }
 
 // The segments as tiles, in as few launches as their descriptors allow.
 // Descriptors are written where the launch reads them; page lists follow.
-// WARP = false: every user address is 16-byte aligned, and tiles_fit.
+// WARP = false: every user address is 16-byte aligned, and every tile lies in
+// one page or run.
 template <Mode M, bool WARP>
-t2i_status Store::launch_tiles(const std::vector<Seg>& segs, cudaStream_t stream) {
+t2i_status TileLauncher::launch_tiles(const std::vector<Seg>& segs, cudaStream_t stream) {
     constexpr uint64_t kTile = WARP ? kWarpTileBytes : kTileBytes;
     TileSeg* const out = reinterpret_cast<TileSeg*>(param_buf_ + sizeof(TileHeader));
     uint32_t n_seg = 0, tiles = 0;
@@ -63,10 +111,10 @@ t2i_status Store::launch_tiles(const std::vector<Seg>& segs, cudaStream_t stream
     auto flush = [&]() -> t2i_status {
         const size_t bytes = n_seg * sizeof(TileSeg) + lp_.size() * sizeof(uint32_t);
         const t2i_status st = n_seg == 0                    ? T2I_OK
-                              : bytes <= size_t(kBlobTiny)  ? launch_tiles_one<M, WARP, kBlobTiny>(n_seg, tiles, stream)
-                              : bytes <= size_t(kBlobSmall) ? launch_tiles_one<M, WARP, kBlobSmall>(n_seg, tiles, stream)
-                              : bytes <= size_t(kBlobMid)   ? launch_tiles_one<M, WARP, kBlobMid>(n_seg, tiles, stream)
-                                                            : launch_tiles_one<M, WARP, kBlobLarge>(n_seg, tiles, stream);
+                              : bytes <= size_t(kBlobTiny)  ? launch_one<M, WARP, kBlobTiny>(n_seg, tiles, stream)
+                              : bytes <= size_t(kBlobSmall) ? launch_one<M, WARP, kBlobSmall>(n_seg, tiles, stream)
+                              : bytes <= size_t(kBlobMid)   ? launch_one<M, WARP, kBlobMid>(n_seg, tiles, stream)
+                                                            : launch_one<M, WARP, kBlobLarge>(n_seg, tiles, stream);
         n_seg = tiles = 0;
         lp_.clear();
         return st;
@@ -108,7 +156,7 @@ t2i_status Store::launch_tiles(const std::vector<Seg>& segs, cudaStream_t stream
 // Aligned segments that fit CTA tiles run as those; the rest of the call, or
 // all of it, is one launch of warp tiles.
 template <Mode M>
-t2i_status Store::launch_segments(const std::vector<Seg>& segs, cudaStream_t stream) {
+t2i_status TileLauncher::launch(const std::vector<Seg>& segs, cudaStream_t stream) {
     uint64_t bytes = 0, tiles = 0;
     uint32_t n_other = 0;
     bool fit = true;  // every aligned segment's tiles lie in one page or run

@@ -105,12 +105,15 @@ int log2_exact(uint64_t v) {
 
 }  // namespace
 
+#include "launch.cuh"
+
 // -------------------------------------------------------------------- Store
 class Store {
   public:
     Store(void* pool, const t2i_store_config& cfg, int device)
         : pool_(reinterpret_cast<uint64_t>(pool)), cfg_(cfg), device_(device),
-          ctl_(cfg.pool_bytes / cfg.page_bytes, cfg.page_bytes, cfg.alloc_policy) {
+          ctl_(cfg.pool_bytes / cfg.page_bytes, cfg.page_bytes, cfg.alloc_policy),
+          launcher_(pool_, uint32_t(log2_exact(cfg.page_bytes)), &ctl_.counters().launches) {
         handle_.core = &ctl_;
         handle_.owned = false;
         handle_.mu = &mu;
@@ -128,7 +131,7 @@ class Store {
     Control& ctl() { return ctl_; }
     const std::string& error() const { return err_; }
     void set_error(std::string e) { err_ = std::move(e); }
-    void inject_launch_failure(uint32_t countdown) { fail_countdown_ = countdown; }
+    void inject_launch_failure(uint32_t countdown) { launcher_.fail_countdown = countdown; }
 
     t2i_status put(const t2i_put_desc* descs, uint32_t n, t2i_id* ids, cudaStream_t stream);
     t2i_status get(const t2i_get_desc* descs, uint32_t n, t2i_status* per_item, cudaStream_t stream,
@@ -154,24 +157,12 @@ class Store {
         return n && a < pend && pool_ < a + n;
     }
 
-    // ---- launch building
-    struct Seg {
-        uint64_t user;
-        uint64_t nbytes_flags;
-        const uint32_t* pages;
-        uint32_t n_pages;
-    };
+    // ---- launches of segs_
     template <Mode M>
-    t2i_status launch_segments(const std::vector<Seg>& segs, cudaStream_t stream);
-    t2i_status launch_kernel(const void* fn, unsigned grid, unsigned threads, cudaStream_t stream);
-    template <Mode M, bool WARP>
-    t2i_status launch_tiles(const std::vector<Seg>& segs, cudaStream_t stream);
-    template <Mode M, bool WARP, int BLOB>
-    t2i_status launch_tiles_one(uint32_t n_seg, uint32_t n_tiles, cudaStream_t stream);
-    static bool pages_are_run(const Seg& s) {
-        for (uint32_t k = 1; k < s.n_pages; ++k)
-            if (s.pages[k] != s.pages[0] + k) return false;
-        return true;
+    t2i_status launch_segments(cudaStream_t stream) {
+        const t2i_status st = launcher_.launch<M>(segs_, stream);
+        if (st != T2I_OK) err_ = launcher_.error;
+        return st;
     }
     // the call's stream in the dependency tracker (creating its events)
     t2i_status stream_slot(cudaStream_t s, int* si) {
@@ -193,11 +184,7 @@ class Store {
     Control ctl_;
     t2i_ctl handle_{};
     uint32_t page_shift_ = 0;
-    uint32_t fail_countdown_ = 0;  // > 0: that many launches from now, report a failure (testing)
-    // TileHeader::flags of the current call's launches: kPrefetchSources
-    // unless a put reads host or managed memory
-    uint32_t launch_flags_ = kPrefetchSources;
-    std::vector<Seg> aligned_, general_;
+    TileLauncher launcher_;
     StreamDeps deps_;
     std::string err_;
     std::vector<const Object*> objs_;
@@ -210,8 +197,6 @@ class Store {
 #endif
     static constexpr size_t kCompactFirstBatch = T2I_TUNE_COMPACT_FIRST;  // moves in the first launch
     static_assert(kMovesPerLaunch * sizeof(TileSeg) <= size_t(kBlobLarge), "moves per launch");
-    std::vector<uint32_t> lp_;
-    alignas(16) unsigned char param_buf_[sizeof(TileParams<kBlobLarge>)];
 };
 
 t2i_status Store::check_user(const void* p, uint64_t n, bool want_write, bool is_host_flag, uint64_t* dev_addr,
@@ -280,8 +265,6 @@ t2i_status Store::check_user(const void* p, uint64_t n, bool want_write, bool is
     }
     return T2I_OK;
 }
-
-#include "launch.cuh"
 
 t2i_status Store::put(const t2i_put_desc* descs, uint32_t n, t2i_id* ids, cudaStream_t stream) {
     if (n == 0) return T2I_OK;
@@ -381,9 +364,9 @@ t2i_status Store::put(const t2i_put_desc* descs, uint32_t n, t2i_id* ids, cudaSt
         }
     }
     if (!segs_.empty()) {
-        launch_flags_ = device_sources ? kPrefetchSources : 0;
-        st = launch_segments<Mode::Put>(segs_, stream);
-        launch_flags_ = kPrefetchSources;
+        launcher_.flags = device_sources ? kPrefetchSources : 0;
+        st = launch_segments<Mode::Put>(stream);
+        launcher_.flags = kPrefetchSources;
         if (st != T2I_OK) {
             mark_writes();
             ctl_.rollback_put(ids, n);
@@ -471,7 +454,7 @@ t2i_status Store::get(const t2i_get_desc* descs, uint32_t n, t2i_status* per_ite
     if (any) {
         cudaError_t we = deps_.wait();
         if (we != cudaSuccess) return cuda_fail("get: cannot order after earlier calls", we);
-        st = segs_.empty() ? T2I_OK : launch_segments<Mode::Get>(segs_, stream);
+        st = segs_.empty() ? T2I_OK : launch_segments<Mode::Get>(stream);
         // items for the copy engine (pinned host destinations, d2h_mode = 1):
         // one copy per run of consecutive pages
         const uint64_t P = uint64_t(1) << page_shift_;
@@ -609,7 +592,7 @@ t2i_status Store::pull_from(Store& src, const t2i_id* ids, uint32_t n, uint32_t 
         return cuda_fail("pull: cannot order after earlier calls", we);
     }
     if (!segs_.empty()) {
-        st = launch_segments<Mode::Move>(segs_, stream);
+        st = launch_segments<Mode::Move>(stream);
         // marked even after a failure part-way: launches before it may still
         // be reading the sources and writing the pages handed back
         uint32_t qd = 0, qs = 0;
@@ -701,7 +684,7 @@ t2i_status Store::pull_pages(const void* src_pool, uint64_t src_pool_bytes, cons
         ctl_.rollback_put(out_ids, n);
         return cuda_fail("pull_pages: cannot order after earlier calls", we);
     }
-    st = launch_segments<Mode::Move>(segs_, stream);
+    st = launch_segments<Mode::Move>(stream);
     // marked even after a failure part-way: launches before it may still be
     // writing the pages handed back
     uint32_t q = 0;
@@ -760,7 +743,7 @@ t2i_status Store::compact(uint64_t limit_bytes, cudaStream_t stream, uint64_t* m
         // each move is a one-page segment whose source is the old page
         for (const t2i_move& m : batch_)
             segs_.push_back({pool_ + uint64_t(m.src_page) * P, m.valid_bytes, &m.dst_page, 1u});
-        st = launch_segments<Mode::Move>(segs_, stream);
+        st = launch_segments<Mode::Move>(stream);
         // marked even after a failure: launches before it may still be
         // reading the old pages and writing the new ones
         uint32_t q = 0;
@@ -979,119 +962,43 @@ const char* t2i_last_error(const t2i_store* store) {
 }  // extern "C"
 
 // ================================================= gather without allocation
-// t2i_gather_noalloc: the chunked gather of one object's pages for callers
-// that cannot allocate device memory (see include/t2istore.h). Its chunk
-// counters live in a file-scope array that is part of the library's device
-// image, so the call allocates nothing. The paper has no counterpart.
+// t2i_gather_noalloc: the gather of one object's pages for callers that
+// cannot allocate device memory (see include/t2istore.h). Its launches are
+// those of a one-item get: tiles need no memory but the launch's parameters.
+// The paper has no counterpart.
 namespace t2i {
 namespace {
-constexpr uint32_t kNoAllocCounters = 64;  // one per launch of a call: 2 KiB in all
-constexpr uint64_t kNoAllocMaxPagesPerLaunch = (kBlobLarge - sizeof(SegDesc)) / sizeof(uint32_t);
-// pages per launch: the page list fits the parameters and the bytes fit
-// 32-bit granule offsets
+constexpr uint64_t kNoAllocMaxLaunches = 64;
+constexpr uint64_t kNoAllocMaxPagesPerLaunch = (kBlobLarge - sizeof(TileSeg)) / sizeof(uint32_t);
+// the most pages of a call: 64 launches of scattered pages, at most 64 GiB each
 uint64_t noalloc_pages_per_launch(uint64_t page_bytes) {
-    return std::min<uint64_t>(kNoAllocMaxPagesPerLaunch, std::max<uint64_t>(1, kMaxSegBytes / page_bytes));
+    return std::min<uint64_t>(kNoAllocMaxPagesPerLaunch, std::max<uint64_t>(1, (uint64_t(1) << 36) / page_bytes));
+}
+
+// Loads every gather kernel on the current device (the driver loads a kernel,
+// allocating device memory for it, when it is first named), once per device:
+// later calls then allocate nothing and can be captured.
+template <int... BLOB>
+cudaError_t load_gathers() {
+    cudaFuncAttributes a;
+    cudaError_t e = cudaSuccess;
+    for (const void* fn : {tile_kernel<Mode::Get, false, BLOB>()..., tile_kernel<Mode::Get, true, BLOB>()...})
+        if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, fn);
+    return e;
 }
 constexpr int kNoAllocMaxDevices = 64;
-}  // namespace
-}  // namespace t2i
-
-// Every GPU that loads the library holds this array until the process exits.
-static __device__ __align__(256) t2i::WorkCounter t2i_noalloc_scratch[t2i::kNoAllocCounters];
-
-namespace t2i {
-namespace {
-
-// The kernels a call can run, as a store's chunked get picks them: the
-// cast-capable gather for 16-byte aligned destinations and for casts, the
-// copy-only gather for other destinations without a cast.
-enum NoAllocKernel { kNoAllocGetAligned = 0, kNoAllocGetAny = 1, kNoAllocCopyAny = 2 };
-
-// Per-device set-up, done once by the first call on that device: the
-// device address of the scratch array (host code sees only a stand-in for
-// the symbol) and the resident CTAs of the gather kernels (its grid size).
-struct NoAllocDevice {
-    bool ready = false;
-    WorkCounter* scratch = nullptr;
-    int max_ctas[3] = {1, 1, 1};  // [NoAllocKernel]
-};
-
-const void* noalloc_kernel(int k) {
-    return k == kNoAllocGetAligned ? reinterpret_cast<const void*>(gather_get_kernel<kBlobLarge, false>)
-           : k == kNoAllocGetAny   ? reinterpret_cast<const void*>(gather_get_kernel<kBlobLarge, true>)
-                                   : reinterpret_cast<const void*>(gather_copy_kernel<kBlobLarge, true>);
-}
-
 std::mutex g_noalloc_mu;
-NoAllocDevice g_noalloc_dev[kNoAllocMaxDevices];
+bool g_noalloc_loaded[kNoAllocMaxDevices];
 
-t2i_status noalloc_setup(int device, NoAllocDevice** out) {
+t2i_status noalloc_setup(int device) {
     std::lock_guard<std::mutex> lock(g_noalloc_mu);
-    NoAllocDevice& d = g_noalloc_dev[device];
-    if (!d.ready) {
-        DeviceGuard g(device);
-        void* ptr = nullptr;
-        cudaError_t e = cudaGetSymbolAddress(&ptr, t2i_noalloc_scratch);
-        if (e != cudaSuccess || !ptr) {
-            set_thread_error(std::string("t2i_gather_noalloc: cannot get the scratch array's device address: ") +
-                             cudaGetErrorString(e));
-            return T2I_ERR_CUDA;
-        }
-        int sms = 0;
-        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess || sms <= 0) {
-            set_thread_error("t2i_gather_noalloc: cannot query the device");
-            return T2I_ERR_CUDA;
-        }
-        for (int k = 0; k < 3; ++k) {
-            int occ = 0;
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, noalloc_kernel(k), kThreads, 0);
-            d.max_ctas[k] = sms * (occ > 0 ? occ : 1);
-        }
-        d.scratch = static_cast<WorkCounter*>(ptr);
-        d.ready = true;
-    }
-    *out = &d;
-    return T2I_OK;
-}
-
-// One launch of kernel `kern`: `np` pages of the object starting at page
-// index `p0`.
-t2i_status noalloc_one(const NoAllocDevice& d, int kern, uint32_t k, const void* pool, int shift,
-                       const uint32_t* pages, uint64_t p0, uint64_t np, uint64_t nbytes, unsigned char* dst, bool cast,
-                       cudaStream_t stream) {
-    thread_local LaunchParams<kBlobLarge> p;  // host-side parameter staging (no device memory)
-    const uint64_t P = uint64_t(1) << shift;
-    const uint64_t off = p0 * P;
-    const uint64_t seg_bytes = std::min<uint64_t>(nbytes - off, np * P);
-    p.h.pool = reinterpret_cast<uint64_t>(pool);
-    p.h.work = reinterpret_cast<uint64_t>(d.scratch + k);
-    p.h.n_seg = 1;
-    p.h.n_granules = static_cast<uint32_t>((seg_bytes + kGranule - 1) / kGranule);
-    p.h.page_shift = static_cast<uint32_t>(shift);
-    p.h.piece_bytes = static_cast<uint32_t>(std::min<uint64_t>(kPieceBytes, P));
-    p.h.pages_offset = sizeof(SegDesc);
-    p.h.chunk_granules = kChunkGranules;
-    p.h.flags = 0;
-    p.h.prefetch_ctas = 0;
-    SegDesc s;
-    s.user = reinterpret_cast<uint64_t>(dst) + (cast ? off / 2 : off);
-    s.nbytes_flags = seg_bytes | (cast ? kCastFlag : 0);
-    s.start = 0;
-    s.page_begin = 0;
-    std::memcpy(p.blob, &s, sizeof(s));
-    std::memcpy(p.blob + sizeof(SegDesc), pages + p0, np * sizeof(uint32_t));
-    const uint64_t want = (seg_bytes + kMinCtaBytes - 1) / kMinCtaBytes;
-    const unsigned grid = static_cast<unsigned>(std::max<uint64_t>(1, std::min<uint64_t>(want, uint64_t(d.max_ctas[kern]))));
-    cudaLaunchConfig_t lc = {};
-    lc.gridDim = dim3(grid);
-    lc.blockDim = dim3(kThreads);
-    lc.stream = stream;
-    void* args[] = {&p};
-    cudaError_t e = cudaLaunchKernelExC(&lc, noalloc_kernel(kern), args);
+    if (g_noalloc_loaded[device]) return T2I_OK;
+    const cudaError_t e = load_gathers<kBlobTiny, kBlobSmall, kBlobMid, kBlobLarge>();
     if (e != cudaSuccess) {
-        set_thread_error(std::string("t2i_gather_noalloc: kernel launch failed: ") + cudaGetErrorString(e));
+        set_thread_error(std::string("t2i_gather_noalloc: cannot load the kernels: ") + cudaGetErrorString(e));
         return T2I_ERR_CUDA;
     }
+    g_noalloc_loaded[device] = true;
     return T2I_OK;
 }
 
@@ -1117,11 +1024,11 @@ extern "C" t2i_status t2i_gather_noalloc(const void* pool_dev, uint64_t pool_byt
             return T2I_ERR_INVALID;
         }
         const uint64_t per_launch = noalloc_pages_per_launch(page_bytes);
-        const uint64_t max_pages = uint64_t(kNoAllocCounters) * per_launch;
+        const uint64_t max_pages = kNoAllocMaxLaunches * per_launch;
         if (n_pages > max_pages) {
             set_thread_error("t2i_gather_noalloc: " + std::to_string(n_pages) + " pages exceed the maximum of " +
-                             std::to_string(max_pages) + " (" + std::to_string(kNoAllocCounters) +
-                             " launches of " + std::to_string(per_launch) + " pages, one scratch counter each)");
+                             std::to_string(max_pages) + " (" + std::to_string(kNoAllocMaxLaunches) +
+                             " launches of " + std::to_string(per_launch) + " pages)");
             return T2I_ERR_INVALID;
         }
         if (nbytes == 0) return T2I_OK;
@@ -1162,28 +1069,14 @@ extern "C" t2i_status t2i_gather_noalloc(const void* pool_dev, uint64_t pool_byt
             set_thread_error("t2i_gather_noalloc: the destination overlaps the pool");
             return T2I_ERR_INVALID;
         }
-        NoAllocDevice* d = nullptr;
-        t2i_status st = noalloc_setup(device, &d);
-        if (st != T2I_OK) return st;
         DeviceGuard g(device);
-        cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
-        const uint64_t n_launch = (n_pages + per_launch - 1) / per_launch;
-        // the counters this call uses start at zero whatever an earlier call left
-        cudaError_t e = cudaMemsetAsync(d->scratch, 0, n_launch * sizeof(WorkCounter), stream);
-        if (e != cudaSuccess) {
-            set_thread_error(std::string("t2i_gather_noalloc: cannot clear the scratch counters: ") +
-                             cudaGetErrorString(e));
-            return T2I_ERR_CUDA;
-        }
-        const int kern = (da & 15u) == 0 ? kNoAllocGetAligned : cast ? kNoAllocGetAny : kNoAllocCopyAny;
-        unsigned char* dst = static_cast<unsigned char*>(dst_dev);
-        for (uint64_t k = 0; k < n_launch; ++k) {
-            const uint64_t p0 = k * per_launch;
-            const uint64_t np = std::min<uint64_t>(per_launch, n_pages - p0);
-            st = noalloc_one(*d, kern, uint32_t(k), pool_dev, shift, pages, p0, np, nbytes, dst, cast != 0, stream);
-            if (st != T2I_OK) return st;
-        }
-        return T2I_OK;
+        const t2i_status st = noalloc_setup(device);
+        if (st != T2I_OK) return st;
+        TileLauncher launcher(pa, uint32_t(shift), nullptr);
+        const std::vector<Seg> segs{{da, nbytes | (cast ? kCastFlag : 0), pages, n_pages}};
+        const t2i_status ls = launcher.launch<Mode::Get>(segs, static_cast<cudaStream_t>(cuda_stream));
+        if (ls != T2I_OK) set_thread_error("t2i_gather_noalloc: " + launcher.error);
+        return ls;
     } catch (const std::exception& ex) {
         set_thread_error(std::string("t2i_gather_noalloc: host error: ") + ex.what());
         return T2I_ERR_INVALID;

@@ -407,9 +407,7 @@ def gather_noalloc(pool, page_bytes: int, pages, nbytes: int, dst, dst_bytes: in
                    stream=None, device: int | None = None, pool_bytes: int | None = None) -> int:
     """t2i_gather_noalloc: one object's pages (``pages``, indices into
     ``pool``) gathered into ``dst`` with no store and no allocation, for
-    callers that cannot allocate device memory. Returns the status; every
-    call shares the library's static scratch counters, so calls that overlap
-    on the GPU race."""
+    callers that cannot allocate device memory. Returns the status."""
     lib = L.load()
     pg = np.ascontiguousarray(pages, dtype=np.uint32)
     if device is None:

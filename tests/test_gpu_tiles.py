@@ -8,7 +8,7 @@ import pytest
 import torch
 
 from oracle.cast import f32_bits_to_bf16_bits
-from paper_2607_26566_gb300 import Store, get_descs, put_descs
+from paper_2607_26566_gb300 import Store, gather_noalloc, get_descs, put_descs
 
 pytestmark = pytest.mark.gpu
 DEV = torch.device("cuda", 0)
@@ -95,3 +95,36 @@ def test_warp_tiles_at_their_edges(P, mis):
             h = o.cpu().numpy()
             assert np.array_equal(h[mis:mis + w.size], w), n
             assert (h[:mis] == 0xCD).all() and (h[mis + w.size:] == 0xCD).all(), n
+
+
+def test_gather_without_a_store_overlapping_and_captured():
+    """gather_noalloc on four streams at once (no shared scratch), and captured
+    into a CUDA graph after a kernel and after a copy that write its pool:
+    every byte as the input's."""
+    P, n = 65536, 9 << 20
+    pages = np.random.default_rng(2).permutation(400)[:n // P].astype(np.uint32)
+    pool = torch.randint(0, 256, (400 * P,), dtype=torch.uint8, device=DEV)
+    want = pool.view(400, P)[torch.from_numpy(pages.astype(np.int64)).to(DEV)].reshape(-1)
+    outs = [torch.zeros(n + 8, dtype=torch.uint8, device=DEV) for _ in range(4)]
+    streams = [torch.cuda.Stream() for _ in range(4)]
+    torch.cuda.synchronize()
+    for _ in range(8):
+        for k, (o, s) in enumerate(zip(outs, streams)):
+            assert gather_noalloc(pool, P, pages, n, o.data_ptr() + k, dst_bytes=n, stream=s) == 0
+    torch.cuda.synchronize()
+    for k, o in enumerate(outs):
+        assert torch.equal(o[k:k + n], want)
+    src = pool.clone()
+    out_a, out_b = torch.zeros(n, dtype=torch.uint8, device=DEV), torch.zeros(n, dtype=torch.uint8, device=DEV)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        pool.bitwise_xor_(255)
+        assert gather_noalloc(pool, P, pages, n, out_a) == 0
+        pool.copy_(src)
+        assert gather_noalloc(pool, P, pages, n, out_b) == 0
+    for _ in range(3):
+        out_a.zero_()
+        out_b.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(out_a, want ^ 255) and torch.equal(out_b, want)
