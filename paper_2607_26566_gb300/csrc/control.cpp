@@ -130,7 +130,9 @@ Control::Control(uint64_t total_pages, uint64_t page_bytes, uint32_t policy)
       limit_pages_(total_pages),
       free_(total_pages, policy),
       page_obj_(total_pages, nullptr),
-      page_idx_(total_pages, 0) {}
+      page_idx_(total_pages, 0) {
+    spare_.reserve(kSpare);
+}
 
 void Control::own(const Object* o) {
     for (uint32_t j = 0; j < o->pages.size(); ++j) {
@@ -145,6 +147,23 @@ void Control::disown(const Object* o) {
 
 Control::~Control() {
     for (Object* o : live_) delete o;
+    for (Object* o : spare_) delete o;
+}
+
+Object* Control::new_object() {
+    if (spare_.empty()) return new Object();
+    Object* o = spare_.back();
+    spare_.pop_back();
+    return o;
+}
+
+void Control::drop(Object* o) {
+    if (spare_.size() >= kSpare || o->pages.capacity() > kSparePages) {
+        delete o;
+        return;
+    }
+    o->pages.clear();
+    spare_.push_back(o);
 }
 
 Group* Control::group_for(uint64_t key) {
@@ -205,7 +224,7 @@ void Control::release(Object* o, bool evicted) {
         ids_.set(o->id, IdTable::kEvicted, next_id_);
     else
         ids_.clear(o->id, next_id_);
-    delete o;
+    drop(o);
     maybe_drop_group(g);
 }
 
@@ -268,8 +287,8 @@ t2i_status Control::put(const t2i_put_desc* descs, uint32_t n, t2i_id* ids, std:
         return T2I_ERR_INVALID;
     }
     uint64_t demand = 0;
-    std::vector<uint64_t> pinned;
-    pinned.reserve(n);
+    std::vector<uint64_t>& pinned = pinned_;
+    pinned.clear();
     for (uint32_t i = 0; i < n; ++i) {
         if (descs[i].reserved != 0) {
             err_ = "put: reserved field must be 0";
@@ -283,7 +302,7 @@ t2i_status Control::put(const t2i_put_desc* descs, uint32_t n, t2i_id* ids, std:
             return T2I_ERR_NOSPACE;
         }
         demand += np;
-        pinned.push_back(descs[i].group);
+        if (pinned.empty() || pinned.back() != descs[i].group) pinned.push_back(descs[i].group);
     }
     std::sort(pinned.begin(), pinned.end());
     pinned.erase(std::unique(pinned.begin(), pinned.end()), pinned.end());
@@ -317,21 +336,22 @@ t2i_status Control::put(const t2i_put_desc* descs, uint32_t n, t2i_id* ids, std:
         }
     }
 
+    Group* g = nullptr;
     for (uint32_t i = 0; i < n; ++i) {
         const t2i_put_desc& d = descs[i];
-        Object* o = new Object();
+        Object* o = new_object();
         o->id = next_id_++;
         o->nbytes = d.nbytes;
         o->dtype_tag = d.dtype_tag;
         o->order = d.order;
         o->evictable = d.evictable != 0;
         o->consumers_left = d.consumers;
-        o->group = group_for(d.group);
+        if (!g || g->key != d.group) g = group_for(d.group);
+        o->group = g;
         const uint64_t np = pages_for(d.nbytes);
         free_.take(np, &o->pages);
         own(o);
         used_pages_ += np;
-        Group* g = o->group;
         g->n_objects++;
         if (o->evictable) {
             g->victims.insert({o->order, o->id});
@@ -380,21 +400,20 @@ void Control::rollback_put(const t2i_id* ids, uint32_t n) {
         live_.pop_back();
         ids_.clear(o->id, next_id_);
         if (o->id + 1 == next_id_) next_id_ = o->id;  // never handed out: issue again
-        delete o;
+        drop(o);
         maybe_drop_group(g);
     }
 }
 
-void Control::account_get(const t2i_id* ids, uint32_t n, size_t stride) {
-    const char* base = reinterpret_cast<const char*>(ids);
-    for (uint32_t i = 0; i < n; ++i) {
-        const t2i_id id = *reinterpret_cast<const t2i_id*>(base + i * stride);
-        Object* o = reinterpret_cast<Object*>(ids_.get(id));
-        touch(o);
-        counters_.gets++;
-        counters_.bytes_got += o->nbytes;
-        if (o->consumers_left > 0 && --o->consumers_left == 0) pending_release_.push_back(o);
-    }
+void Control::account(Object* o) {
+    touch(o);
+    counters_.gets++;
+    counters_.bytes_got += o->nbytes;
+    if (o->consumers_left > 0 && --o->consumers_left == 0) pending_release_.push_back(o);
+}
+
+void Control::account_get(const Object* const* objs, uint32_t n) {
+    for (uint32_t i = 0; i < n; ++i) account(const_cast<Object*>(objs[i]));
     flush_touches();
 }
 
@@ -441,7 +460,8 @@ t2i_status Control::get(const t2i_get_desc* descs, uint32_t n, t2i_status* per_i
     if (objs) {
         for (uint32_t i = 0; i < n; ++i) (*objs)[i] = reinterpret_cast<const Object*>(ids_.get(descs[i].id));
     }
-    account_get(&descs[0].id, n, sizeof(t2i_get_desc));
+    for (uint32_t i = 0; i < n; ++i) account(reinterpret_cast<Object*>(ids_.get(descs[i].id)));
+    flush_touches();
     if (!defer_release) release_pending();
     return T2I_OK;
 }

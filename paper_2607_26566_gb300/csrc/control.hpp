@@ -158,7 +158,7 @@ class Control {
     // The accounting half of a get (recency stamps, consumer counts) for
     // items already validated; objects consumed to zero wait for
     // release_pending(). Called after the get's copies are enqueued.
-    void account_get(const t2i_id* ids, uint32_t n, size_t stride);
+    void account_get(const Object* const* objs, uint32_t n);
     // get: validates every item (per_item nullable), then stamps recency and
     // counts consumers. objs[i] receives the object of descs[i] on success.
     // dst fields are not looked at here. Objects whose last consumer this was
@@ -205,6 +205,9 @@ class Control {
     Group* group_for(uint64_t key);
     void maybe_drop_group(Group* g);
     void touch(Object* o);
+    void account(Object* o);
+    Object* new_object();
+    void drop(Object* o);
     void flush_touches();
     void release(Object* o, bool evicted);
 
@@ -219,9 +222,14 @@ class Control {
     FreePages free_;
     IdTable ids_;
     std::vector<Object*> live_;
+    // released objects kept for the next puts (their page lists keep their
+    // memory): at most kSpare of at most kSparePages pages
+    static constexpr size_t kSpare = 1024, kSparePages = 256;
+    std::vector<Object*> spare_;
     std::unordered_map<uint64_t, std::unique_ptr<Group>> groups_;
     std::set<std::pair<uint64_t, Group*>> recency_;   // groups holding evictable objects
     std::vector<Group*> touched_;
+    std::vector<uint64_t> pinned_;   // the groups of the current put, sorted
     std::vector<t2i_id> last_evictions_;
     std::vector<Object*> pending_release_;   // consumed to zero by the last get
     struct Remap {

@@ -44,26 +44,25 @@ class StreamDeps {
 
     void resize_pages(uint64_t n) { pages_.assign(n, PageDeps{}); }
 
-    // Index of `s`, registering it (and its events) on first use. -1 if the
-    // events cannot be created.
+    // Index of `s`, registering it on first use. -1 if an event that the call
+    // will need cannot be created. (Events are created when they are first
+    // recorded: a stream used alone needs none.)
     int stream_index(cudaStream_t s) {
-        for (size_t i = 0; i < streams_.size(); ++i)
-            if (streams_[i].s == s) return static_cast<int>(i);
-        if (streams_.size() >= 0xFFFF) return -1;
-        State st;
-        st.s = s;
-        if (cudaEventCreateWithFlags(&st.lazy, cudaEventDisableTiming) != cudaSuccess) return -1;
-        for (uint32_t k = 0; k < kRing; ++k) {
-            if (cudaEventCreateWithFlags(&st.ring[k], cudaEventDisableTiming) != cudaSuccess) {
-                for (uint32_t j = 0; j < k; ++j) cudaEventDestroy(st.ring[j]);
-                cudaEventDestroy(st.lazy);
-                return -1;
-            }
-            st.ring_seq[k] = 0;
+        size_t i = 0;
+        while (i < streams_.size() && streams_[i].s != s) ++i;
+        if (i == streams_.size()) {
+            if (streams_.size() >= 0xFFFF) return -1;
+            streams_.emplace_back();
+            streams_.back().s = s;
         }
-        streams_.push_back(st);
-        return static_cast<int>(streams_.size() - 1);
+        if (streams_.size() > 1 && ensure(&streams_[i].ring[(streams_[i].seq + 1) % kRing]) != cudaSuccess) return -1;
+        return static_cast<int>(i);
     }
+
+    // Whether a call may depend on another stream's. While one stream alone has
+    // used the store, reads() and writes() find nothing to wait for and need
+    // not be called; the marks are kept for streams to come.
+    bool several() const { return streams_.size() > 1; }
 
     // --- one call on stream index `si`
     void begin(int si) {
@@ -98,7 +97,8 @@ class StreamDeps {
         *seq_out = q;
         if (streams_.size() > 1) {
             const uint32_t k = q % kRing;
-            cudaError_t e = cudaEventRecord(st.ring[k], st.s);
+            cudaError_t e = ensure(&st.ring[k]);
+            if (e == cudaSuccess) e = cudaEventRecord(st.ring[k], st.s);
             if (e != cudaSuccess) return e;
             st.ring_seq[k] = q;
         }
@@ -126,30 +126,34 @@ class StreamDeps {
     void synchronize_all() {
         for (State& st : streams_) {
             if (st.seq == 0) continue;
-            if (cudaEventRecord(st.lazy, st.s) == cudaSuccess) cudaEventSynchronize(st.lazy);
+            if (ensure(&st.lazy) == cudaSuccess && cudaEventRecord(st.lazy, st.s) == cudaSuccess)
+                cudaEventSynchronize(st.lazy);
         }
     }
 
     void release() {
         for (State& st : streams_) {
-            cudaEventDestroy(st.lazy);
-            for (uint32_t k = 0; k < kRing; ++k) cudaEventDestroy(st.ring[k]);
+            if (st.lazy) cudaEventDestroy(st.lazy);
+            for (cudaEvent_t e : st.ring)
+                if (e) cudaEventDestroy(e);
         }
         streams_.clear();
     }
 
-    size_t n_streams() const { return streams_.size(); }
 
   private:
     struct State {
         cudaStream_t s = nullptr;
         uint32_t seq = 0;           // calls enqueued on this stream
-        cudaEvent_t ring[kRing];    // call q's event lives in ring[q % kRing]
-        uint32_t ring_seq[kRing];   // the call each ring event was last recorded for
+        cudaEvent_t ring[kRing] = {};   // call q's event lives in ring[q % kRing]
+        uint32_t ring_seq[kRing] = {};  // the call each ring event was last recorded for
         cudaEvent_t lazy = nullptr; // "everything so far" on this stream
         uint32_t lazy_seq = 0;
     };
 
+    static cudaError_t ensure(cudaEvent_t* e) {
+        return *e ? cudaSuccess : cudaEventCreateWithFlags(e, cudaEventDisableTiming);
+    }
     void note(const Dep& d) {
         if (d.seq == 0 || d.stream == cur_) return;
         if (need_[d.stream] < d.seq) need_[d.stream] = d.seq;
@@ -163,7 +167,8 @@ class StreamDeps {
         const uint32_t k = q % kRing;
         if (st.ring_seq[k] >= q) return cudaStreamWaitEvent(s, st.ring[k], 0);
         if (st.lazy_seq < q) {
-            cudaError_t e = cudaEventRecord(st.lazy, st.s);
+            cudaError_t e = ensure(&st.lazy);
+            if (e == cudaSuccess) e = cudaEventRecord(st.lazy, st.s);
             if (e != cudaSuccess) return e;
             st.lazy_seq = st.seq;
         }

@@ -43,6 +43,24 @@ static int nargs_ok(Py_ssize_t n, Py_ssize_t want, const char* name) {
     return 0;
 }
 
+/* The ids of a uint64 array (native byte order, C-contiguous, n entries or
+ * more along its first axis; n < 0: a one-dimensional array of any length).
+ * Asking the array itself costs a fraction of its ctypes.data attribute. 1:
+ * *view is held; 0: not such an array, no Python error. */
+static int ids_of(PyObject* obj, Py_ssize_t n, Py_buffer* view) {
+    if (!PyObject_CheckBuffer(obj)) return 0;
+    if (PyObject_GetBuffer(obj, view, PyBUF_FORMAT | PyBUF_C_CONTIGUOUS) != 0) {
+        PyErr_Clear();
+        return 0;
+    }
+    const char* f = view->format;
+    if (view->itemsize == 8 && f && (f[0] == 'L' || f[0] == 'Q') && f[1] == '\0' && view->ndim >= 1 &&
+        (n < 0 ? view->ndim == 1 && view->shape[0] <= 0xFFFFFFFF : view->shape[0] >= n))
+        return 1;
+    PyBuffer_Release(view);
+    return 0;
+}
+
 /* put_batch(store, descs, n, out_ids, stream) -> status (t2i_put_batch) */
 static PyObject* py_put_batch(PyObject* self, PyObject* const* args, Py_ssize_t n) {
     void *h, *d, *ids, *s;
@@ -87,6 +105,42 @@ static PyObject* py_get_batch_ids(PyObject* self, PyObject* const* args, Py_ssiz
     return PyLong_FromLong(t2i_get_batch((t2i_store*)h, g, cnt, (t2i_status*)per, s));
 }
 
+/* get_batch_for(store, descs, n, ids, per_item, stream) -> status, or None if
+ * ids is not a uint64 array of n entries or more: get_batch_ids with the
+ * array itself. */
+static PyObject* py_get_batch_for(PyObject* self, PyObject* const* args, Py_ssize_t n) {
+    void *h, *d, *per, *s;
+    uint32_t cnt;
+    Py_buffer view;
+    (void)self;
+    if (!nargs_ok(n, 6, "get_batch_for") || !arg_ptr(args, 0, &h) || !arg_ptr(args, 1, &d) ||
+        !arg_u32(args, 2, &cnt) || !arg_ptr(args, 4, &per) || !arg_ptr(args, 5, &s))
+        return NULL;
+    if (cnt && !d) {
+        PyErr_SetString(PyExc_ValueError, "get_batch_for: null descriptor array");
+        return NULL;
+    }
+    if (!ids_of(args[3], (Py_ssize_t)cnt, &view)) Py_RETURN_NONE;
+    t2i_get_desc* g = (t2i_get_desc*)d;
+    const t2i_id* src = (const t2i_id*)view.buf;
+    for (uint32_t i = 0; i < cnt; ++i) g[i].id = src[i];
+    PyBuffer_Release(&view);
+    return PyLong_FromLong(t2i_get_batch((t2i_store*)h, g, cnt, (t2i_status*)per, s));
+}
+
+/* free_ids(store, ids) -> status, or None if ids is not a one-dimensional
+ * uint64 array: t2i_free of every id in it. */
+static PyObject* py_free_ids(PyObject* self, PyObject* const* args, Py_ssize_t n) {
+    void* h;
+    Py_buffer view;
+    (void)self;
+    if (!nargs_ok(n, 2, "free_ids") || !arg_ptr(args, 0, &h)) return NULL;
+    if (!ids_of(args[1], -1, &view)) Py_RETURN_NONE;
+    const t2i_status st = t2i_free((t2i_store*)h, (const t2i_id*)view.buf, (uint32_t)view.shape[0]);
+    PyBuffer_Release(&view);
+    return PyLong_FromLong(st);
+}
+
 /* free(store, ids, n) -> status (t2i_free) */
 static PyObject* py_free(PyObject* self, PyObject* const* args, Py_ssize_t n) {
     void *h, *ids;
@@ -105,6 +159,10 @@ static PyMethodDef methods[] = {
     {"get_batch_ids", (PyCFunction)(void (*)(void))py_get_batch_ids, METH_FASTCALL,
      "get_batch_ids(store, descs, n, ids, per_item, stream) -> status: sets the descriptors' ids, then "
      "t2i_get_batch"},
+    {"get_batch_for", (PyCFunction)(void (*)(void))py_get_batch_for, METH_FASTCALL,
+     "get_batch_for(store, descs, n, ids, per_item, stream) -> status, or None: get_batch_ids with a uint64 array"},
+    {"free_ids", (PyCFunction)(void (*)(void))py_free_ids, METH_FASTCALL,
+     "free_ids(store, ids) -> status, or None: t2i_free of a uint64 array"},
     {"free", (PyCFunction)(void (*)(void))py_free, METH_FASTCALL, "free(store, ids, n) -> status: t2i_free"},
     {NULL, NULL, 0, NULL}};
 

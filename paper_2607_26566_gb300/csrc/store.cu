@@ -152,6 +152,8 @@ class Store {
     // ---- pointer checks (per call cache of the last allocation seen)
     t2i_status check_user(const void* p, uint64_t n, bool want_write, bool is_host_flag, uint64_t* dev_addr,
                           bool* needs_copy_engine, Range* cache);
+    t2i_status check_item(const t2i_get_desc& d, const Object** obj, uint64_t* dev_dst, bool* ce, Range* cache);
+    t2i_status fail_get(const t2i_get_desc* descs, uint32_t n, t2i_status* per_item);
     bool overlaps_pool(uint64_t a, uint64_t n) const {
         const uint64_t pend = pool_ + cfg_.pool_bytes;
         return n && a < pend && pool_ < a + n;
@@ -187,7 +189,9 @@ class Store {
     TileLauncher launcher_;
     StreamDeps deps_;
     std::string err_;
-    std::vector<const Object*> objs_;
+    std::vector<const Object*> objs_;  // the current call's objects, and per item:
+    std::vector<uint64_t> addr_;       // the device-visible address of a put's source
+    std::vector<uint8_t> use_ce_;      // 1: the copy engine moves it
     std::vector<Seg> segs_;
     std::vector<t2i_move> batch_;  // the moves of one compaction launch
     // moves per compaction launch: one 24-byte descriptor each
@@ -273,8 +277,10 @@ t2i_status Store::put(const t2i_put_desc* descs, uint32_t n, t2i_id* ids, cudaSt
         return T2I_ERR_INVALID;
     }
     // 1. check every source before touching the directory
-    std::vector<uint64_t> dev_src(n);
-    std::vector<uint8_t> use_ce(n);
+    std::vector<uint64_t>& dev_src = addr_;
+    std::vector<uint8_t>& use_ce = use_ce_;
+    dev_src.assign(n, 0);
+    use_ce.assign(n, 0);
     Range cache;
     bool device_sources = true;  // every source the kernel reads is device memory
     for (uint32_t i = 0; i < n; ++i) {
@@ -314,7 +320,8 @@ t2i_status Store::put(const t2i_put_desc* descs, uint32_t n, t2i_id* ids, cudaSt
     bool any = false;
     for (uint32_t i = 0; i < n; ++i) {
         if (!descs[i].src) continue;  // reserved: nothing is written
-        for (uint32_t pg : objs_[i]->pages) deps_.writes(pg);
+        if (deps_.several())
+            for (uint32_t pg : objs_[i]->pages) deps_.writes(pg);
         any = any || !objs_[i]->pages.empty();
     }
     if (!any) return T2I_OK;
@@ -386,51 +393,24 @@ t2i_status Store::get(const t2i_get_desc* descs, uint32_t n, t2i_status* per_ite
         return T2I_ERR_INVALID;
     }
     // 1. directory (ids, evictions, cast rules) without touching the LRU
-    std::vector<t2i_status> per(n, T2I_OK);
-    std::vector<uint64_t> dev_dst(n, 0);
-    std::vector<uint8_t> use_ce(n, 0);
-    t2i_status first = T2I_OK;
-    uint32_t first_i = 0;
+    objs_.resize(n);
+    use_ce_.assign(n, 0);
+    segs_.clear();
     Range cache;
     for (uint32_t i = 0; i < n; ++i) {
-        const t2i_get_desc& d = descs[i];
-        t2i_status s = T2I_OK;
-        const Object* o = ctl_.find(d.id);
-        if (d.cast > 1 || d.reserved != 0) {
-            s = T2I_ERR_INVALID;
-        } else if (!o) {
-            s = ctl_.is_evicted(d.id) ? T2I_ERR_EVICTED : T2I_ERR_NOT_FOUND;
-        } else {
-            const uint64_t out_bytes = d.cast ? o->nbytes / 2 : o->nbytes;
-            if ((d.cast && (o->nbytes % 4 != 0 || (reinterpret_cast<uint64_t>(d.dst) & 1))) ||
-                d.dst_bytes < out_bytes) {
-                s = T2I_ERR_INVALID;
-            } else {
-                bool ce = false;
-                if (check_user(d.dst, out_bytes, true, false, &dev_dst[i], &ce, &cache) != T2I_OK) s = T2I_ERR_INVALID;
-                use_ce[i] = ce && !d.cast;  // the cast runs in the kernel
-            }
-        }
-        per[i] = s;
-        if (s != T2I_OK && first == T2I_OK) {
-            first = s;
-            first_i = i;
-        }
-    }
-    if (first != T2I_OK) {
-        // nothing is written and the LRU is not touched; misses still count
-        std::string why = err_;
-        for (t2i_status s : per) ctl_.counters().misses += s == T2I_ERR_EVICTED;
-        if (per_item) std::copy(per.begin(), per.end(), per_item);
-        static const char* what[] = {"ok", "invalid", "no space", "id not found", "id was evicted", "cuda"};
-        err_ = "get: item " + std::to_string(first_i) + ": " + what[first] +
-               (first == T2I_ERR_INVALID && !why.empty() ? " (" + why + ")" : "");
-        return first;
+        uint64_t dev_dst = 0;
+        bool ce = false;
+        if (check_item(descs[i], &objs_[i], &dev_dst, &ce, &cache) != T2I_OK)
+            return fail_get(descs, n, per_item);
+        const Object* o = objs_[i];
+        if (ce)
+            use_ce_[i] = 1;
+        else if (o->nbytes)
+            segs_.push_back({dev_dst, o->nbytes | (descs[i].cast ? kCastFlag : 0), o->pages.data(),
+                             uint32_t(o->pages.size())});
     }
     // 2. one gather launch for the batch (copies and casts together), after
     //    the calls that wrote its pages and after the caller's event
-    objs_.resize(n);
-    for (uint32_t i = 0; i < n; ++i) objs_[i] = ctl_.find(descs[i].id);
     DeviceGuard g(device_);
     int si = 0;
     t2i_status st = stream_slot(stream, &si);
@@ -439,17 +419,14 @@ t2i_status Store::get(const t2i_get_desc* descs, uint32_t n, t2i_status* per_ite
         cudaError_t e = cudaStreamWaitEvent(stream, wait_event, 0);
         if (e != cudaSuccess) return cuda_fail("get: cannot wait for the event", e);
     }
-    segs_.clear();
     deps_.begin(si);
     bool any = false;
     for (uint32_t i = 0; i < n; ++i) {
         const Object* o = objs_[i];
         if (o->nbytes == 0) continue;
-        for (uint32_t pg : o->pages) deps_.reads(pg);
         any = true;
-        if (use_ce[i]) continue;
-        segs_.push_back({dev_dst[i], o->nbytes | (descs[i].cast ? kCastFlag : 0), o->pages.data(),
-                         uint32_t(o->pages.size())});
+        if (!deps_.several()) break;
+        for (uint32_t pg : o->pages) deps_.reads(pg);
     }
     if (any) {
         cudaError_t we = deps_.wait();
@@ -460,7 +437,7 @@ t2i_status Store::get(const t2i_get_desc* descs, uint32_t n, t2i_status* per_ite
         const uint64_t P = uint64_t(1) << page_shift_;
         for (uint32_t i = 0; i < n && st == T2I_OK; ++i) {
             const Object* o = objs_[i];
-            if (!use_ce[i] || o->nbytes == 0) continue;
+            if (!use_ce_[i] || o->nbytes == 0) continue;
             char* dst = static_cast<char*>(descs[i].dst);
             size_t j = 0;
             while (j < o->pages.size()) {
@@ -492,9 +469,49 @@ t2i_status Store::get(const t2i_get_desc* descs, uint32_t n, t2i_status* per_ite
     //    objects consumed to zero are freed (their pages carry this call as
     //    a reader, so reuse waits for it)
     if (per_item) std::fill(per_item, per_item + n, T2I_OK);
-    ctl_.account_get(&descs[0].id, n, sizeof(t2i_get_desc));
+    ctl_.account_get(objs_.data(), n);
     ctl_.release_pending();
     return st;
+}
+
+// One get item: its object, where the kernel writes it, whether the copy
+// engine does instead. Changes nothing but err_.
+t2i_status Store::check_item(const t2i_get_desc& d, const Object** obj, uint64_t* dev_dst, bool* ce, Range* cache) {
+    *ce = false;
+    if (d.cast > 1 || d.reserved != 0) return T2I_ERR_INVALID;
+    const Object* o = *obj = ctl_.find(d.id);
+    if (!o) return ctl_.is_evicted(d.id) ? T2I_ERR_EVICTED : T2I_ERR_NOT_FOUND;
+    const uint64_t out_bytes = d.cast ? o->nbytes / 2 : o->nbytes;
+    if ((d.cast && (o->nbytes % 4 != 0 || (reinterpret_cast<uint64_t>(d.dst) & 1))) || d.dst_bytes < out_bytes)
+        return T2I_ERR_INVALID;
+    if (check_user(d.dst, out_bytes, true, false, dev_dst, ce, cache) != T2I_OK) return T2I_ERR_INVALID;
+    if (d.cast) *ce = false;  // the cast runs in the kernel
+    return T2I_OK;
+}
+
+// A get with an item that fails: every item's status; nothing is written and
+// the LRU is not touched, but misses count.
+t2i_status Store::fail_get(const t2i_get_desc* descs, uint32_t n, t2i_status* per_item) {
+    t2i_status first = T2I_OK;
+    uint32_t first_i = 0;
+    Range cache;
+    for (uint32_t i = 0; i < n; ++i) {
+        const Object* o = nullptr;
+        uint64_t dev_dst = 0;
+        bool ce = false;
+        const t2i_status s = check_item(descs[i], &o, &dev_dst, &ce, &cache);
+        if (per_item) per_item[i] = s;
+        ctl_.counters().misses += s == T2I_ERR_EVICTED;
+        if (s != T2I_OK && first == T2I_OK) {
+            first = s;
+            first_i = i;
+        }
+    }
+    const std::string why = err_;
+    static const char* what[] = {"ok", "invalid", "no space", "id not found", "id was evicted", "cuda"};
+    err_ = "get: item " + std::to_string(first_i) + ": " + what[first] +
+           (first == T2I_ERR_INVALID && !why.empty() ? " (" + why + ")" : "");
+    return first;
 }
 
 t2i_status Store::view(t2i_id id, cudaStream_t stream, void** ptr, uint64_t* nbytes) {
@@ -610,7 +627,7 @@ t2i_status Store::pull_from(Store& src, const t2i_id* ids, uint32_t n, uint32_t 
             st = cuda_fail("pull: cannot record its event", e1 != cudaSuccess ? e1 : e2);
     }
     // 4. the sources are read like a get (stamps, consumer counts)
-    src.ctl_.account_get(ids, n, sizeof(t2i_id));
+    src.ctl_.account_get(so.data(), n);
     src.ctl_.release_pending();
     return st;
 }
@@ -728,7 +745,7 @@ t2i_status Store::compact(uint64_t limit_bytes, cudaStream_t stream, uint64_t* m
         batch = std::min<size_t>(batch * 4, kMovesPerLaunch);
         if (batch_.empty()) break;
         deps_.begin(si);
-        if (deps_.n_streams() > 1) {  // with one stream there is nothing to wait for
+        if (deps_.several()) {
             for (const t2i_move& m : batch_) {
                 deps_.reads(m.src_page);
                 deps_.writes(m.dst_page);

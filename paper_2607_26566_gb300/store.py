@@ -285,11 +285,12 @@ class Store:
         """t2i_get_batch on a prepared batch, after setting its ids to ``ids``
         (if given: a uint64 array of at least ``p.n`` ids, e.g. the ids a
         prepared put returned); per-item statuses land in ``p.out``."""
-        if self._fast is not None and (ids is None or (isinstance(ids, np.ndarray) and ids.dtype == np.uint64
-                                                       and ids.flags.c_contiguous and len(ids) >= p.n)):
+        if self._fast is not None:
             if ids is None:
                 return self._fast.get_batch(self._hi, p.addr, p.n, p.out_addr, _stream(stream))
-            return self._fast.get_batch_ids(self._hi, p.addr, p.n, ids.ctypes.data, p.out_addr, _stream(stream))
+            st = self._fast.get_batch_for(self._hi, p.addr, p.n, ids, p.out_addr, _stream(stream))
+            if st is not None:
+                return st
         if ids is not None:
             p.descs["id"] = ids
         return self._lib.t2i_get_batch(self._h, p.addr, p.n, p.out_addr, _stream(stream))
@@ -310,6 +311,10 @@ class Store:
         return st, per
 
     def free(self, ids) -> int:
+        if self._fast is not None:
+            st = self._fast.free_ids(self._hi, ids)
+            if st is not None:
+                return st
         ids = np.ascontiguousarray(ids, np.uint64)
         return self._lib.t2i_free(self._h, ids.ctypes.data, len(ids))
 
