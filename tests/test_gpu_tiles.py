@@ -128,3 +128,27 @@ def test_gather_without_a_store_overlapping_and_captured():
         graph.replay()
         torch.cuda.synchronize()
         assert torch.equal(out_a, want ^ 255) and torch.equal(out_b, want)
+
+
+@pytest.mark.parametrize("P", [65536, 1 << 20])
+@pytest.mark.parametrize("n", [(48 << 20) - 16, (48 << 20) + 20])
+def test_large_calls_of_a_store_used_on_two_streams(P, n):
+    """Calls on both sides of the line between warp and CTA tiles that a store
+    used on several streams has, in scattered pages below and at the page size
+    where it lies: copy and cast, byte for byte."""
+    n_pages = -(-n // P)
+    st = Store(torch.zeros(2 * n_pages * P, dtype=torch.uint8, device=DEV), P)
+    scatter(st, 2 * n_pages, P, 7)
+    f = torch.randn(n // 4, device=DEV)
+    outs = [torch.zeros(n, dtype=torch.uint8, device=DEV), torch.zeros(n // 2, dtype=torch.uint8, device=DEV)]
+    torch.cuda.synchronize()
+    for s in (torch.cuda.Stream(), torch.cuda.Stream()):
+        st_, ids = st.put_batch(put_descs([f]), stream=s)
+        assert st_ == 0
+        assert st.get_batch(get_descs([ids[0], ids[0]], outs, cast=[0, 1]), stream=s)[0] == 0
+        torch.cuda.synchronize()
+        assert torch.equal(outs[0], f.view(torch.uint8))
+        assert torch.equal(outs[1].view(torch.bfloat16), f.to(torch.bfloat16))
+        outs[0].zero_()
+        outs[1].zero_()
+        torch.cuda.synchronize()
