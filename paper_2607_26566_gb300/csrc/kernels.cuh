@@ -55,39 +55,44 @@ constexpr int kBlobLarge = 31 * 1024;  // header + blob stays below the 32,764-b
 // 94.1 / 810 / 755 / 895; 1024 x 2 94.6 / 810 / 765 / 901; 512 x 4 98.2 / 814 /
 // 759 / 904; 256 x 4 96.7 / 815 / 760 / 904; 256 x 2 95.1 / 812 / 757 / 900;
 // 128 x 4 93.9 / 815 / 760 / 904. Without the L2 prefetch: 102.0 / 811 / 757 / 902.
-#ifndef T2I_TUNE_TILE_THREADS
-#define T2I_TUNE_TILE_THREADS 512
-#endif
-#ifndef T2I_TUNE_TILE_VEC
-#define T2I_TUNE_TILE_VEC 2
-#endif
-#ifndef T2I_TUNE_TILE_BLOCKS
-#define T2I_TUNE_TILE_BLOCKS 4
-#endif
+constexpr uint32_t kTileShift = 14;
+constexpr uint32_t kTileBytes = 1u << kTileShift;
+constexpr unsigned kTileThreads = 512;
 #ifndef T2I_TUNE_TILE_MIN_BYTES
 #define T2I_TUNE_TILE_MIN_BYTES (4ull << 20)
 #endif
-constexpr int kTileThreads = T2I_TUNE_TILE_THREADS;
-constexpr int kTileVec = T2I_TUNE_TILE_VEC;
-constexpr uint32_t kTileBytes = kTileThreads * kTileVec * 16;  // 16 KiB
-constexpr uint32_t kTileShift = kTileBytes == 8192 ? 13 : kTileBytes == 16384 ? 14 : kTileBytes == 32768 ? 15 : 16;
-static_assert(kTileBytes == 1u << kTileShift, "tile size");
+// Threads of a launch whose tiles fit the SMs at once, by tiles per SM: as many
+// as leave an SM room for just these CTAs (2,048 threads). With room to
+// spare, the next grid's CTAs fill some SMs early and others late, and its
+// slowest SM decides: eight B=1 requests on one stream (11.5 MB, 705 tiles a
+// call) took 62.4 us a pass in 512 threads, 58.0 in 384; of 14 MB (870) 74.7,
+// 70.0 in 320; a launch of over 8 tiles an SM takes 512.
+#ifndef T2I_TUNE_TILE_BALANCE
+#define T2I_TUNE_TILE_BALANCE 1
+#endif
+constexpr unsigned kTileWaveThreads[] = {1024, 1024, 1024, 672, 512, 384, 320, 288, 256};
+constexpr unsigned kTileMaxPerSm = T2I_TUNE_TILE_BALANCE ? 8 : 0;
+// vectors per thread V: T x V >= 1,024 vectors a tile
+template <int V>
+constexpr unsigned kTileMaxThreads = V == 2 ? 1024 : 384;
 // Aligned launches of at least this many bytes run as CTA tiles, others as
-// warp tiles. The line is broad: put + get of B=4 requests (45 MB a call) took
-// 93.9 us a pass in CTA tiles and 95.3 in warp tiles, of B=1 requests (11.5
-// MB) 69 in both, a 40 MB adapter get 12.2 and 12.0. Below it the launch is
-// bound by its latency, and a warp starts sooner than 512 threads.
+// warp tiles. On one stream eight B=1 requests took (us a pass) 47.1 in CTA
+// tiles and 59.7 in warp tiles at 7 MB a call, 58.0 and 59.3 at 11.5 MB, four
+// of 39 MB 94.1 and 95.3. Below the line the host issues a call in the time
+// that either kernel takes (4 MB: 42.9 and 43.5), and calls of many small
+// segments are the usual ones.
 constexpr uint64_t kTileMinBytes = T2I_TUNE_TILE_MIN_BYTES;
 
-// Warp tiles (see warp_tile): 4 KiB each, one warp each, any alignment. CTAs
-// of 2, 4 or 8 warps ran alike (within 2%) on small and ragged batches.
-#ifndef T2I_TUNE_WARP_THREADS
-#define T2I_TUNE_WARP_THREADS 128
+// Warp tiles (see warp_tile): 4 KiB each, one warp each, any alignment. A
+// launch that fits runs one CTA an SM, of as many warps (up to 32) as share its
+// tiles out evenly; a larger one CTAs of 4 warps. With 4 warps a CTA, eight B=1
+// requests in warp tiles took 68.2 us a pass, evenly shared 59.3 (11.5 MB a
+// call); 14 MB 75.8 and 69.5.
+#ifndef T2I_TUNE_WARP_BALANCE
+#define T2I_TUNE_WARP_BALANCE 1
 #endif
-#ifndef T2I_TUNE_WARP_BLOCKS
-#define T2I_TUNE_WARP_BLOCKS 8
-#endif
-constexpr int kWarpThreads = T2I_TUNE_WARP_THREADS;
+constexpr unsigned kWarpThreads = 128;
+constexpr unsigned kWarpMaxPerSm = T2I_TUNE_WARP_BALANCE ? 32 : 0;  // warps of one CTA
 constexpr int kWarpVec = 8;  // 16-byte source vectors per lane
 constexpr uint32_t kWarpTileShift = 12;
 constexpr uint32_t kWarpTileBytes = 1u << kWarpTileShift;
@@ -176,21 +181,23 @@ __device__ __forceinline__ uint32_t pack_bf16x2(uint32_t a, uint32_t b) {
 #endif
 }
 
-// The copy of one tile (len <= kTileBytes, both sides 16-byte aligned).
+// The copy of one tile by the CTA's threads (len <= kTileBytes <= blockDim.x *
+// V vectors, both sides 16-byte aligned).
+template <int V>
 __device__ __forceinline__ void tile_copy_bytes(unsigned char* __restrict__ dst, const unsigned char* __restrict__ src,
                                                 uint32_t len) {
     const uint32_t nvec = len >> 4;
     const uint4* s = reinterpret_cast<const uint4*>(src);
     uint4* d = reinterpret_cast<uint4*>(dst);
-    uint4 r[kTileVec];
+    uint4 r[V];
 #pragma unroll
-    for (int j = 0; j < kTileVec; ++j) {
-        const uint32_t v = j * kTileThreads + threadIdx.x;
+    for (int j = 0; j < V; ++j) {
+        const uint32_t v = j * blockDim.x + threadIdx.x;
         if (v < nvec) r[j] = ld_stream(s + v);
     }
 #pragma unroll
-    for (int j = 0; j < kTileVec; ++j) {
-        const uint32_t v = j * kTileThreads + threadIdx.x;
+    for (int j = 0; j < V; ++j) {
+        const uint32_t v = j * blockDim.x + threadIdx.x;
         if (v < nvec) st_stream(d + v, r[j]);
     }
     const uint32_t at = (nvec << 4) + threadIdx.x;
@@ -199,25 +206,25 @@ __device__ __forceinline__ void tile_copy_bytes(unsigned char* __restrict__ dst,
 
 // The same with the cast: len source bytes, a multiple of 4. Blocks of 8
 // floats (two 16-byte loads, one 16-byte store), the last < 8 one by one.
+template <int V>
 __device__ __forceinline__ void tile_cast(unsigned char* __restrict__ dst, const unsigned char* __restrict__ src,
                                           uint32_t len) {
-    static_assert(kTileVec % 2 == 0, "a block is two vectors");
+    static_assert(V % 2 == 0, "a block is two vectors");
     const uint32_t n8 = len >> 5;
     const uint4* s = reinterpret_cast<const uint4*>(src);
     uint4* d = reinterpret_cast<uint4*>(dst);
-    constexpr int kSteps = kTileVec / 2;
-    uint4 a[kSteps], b[kSteps];
+    uint4 a[V / 2], b[V / 2];
 #pragma unroll
-    for (int j = 0; j < kSteps; ++j) {
-        const uint32_t v = j * kTileThreads + threadIdx.x;
+    for (int j = 0; j < V / 2; ++j) {
+        const uint32_t v = j * blockDim.x + threadIdx.x;
         if (v < n8) {
             a[j] = ld_stream(s + 2 * v);
             b[j] = ld_stream(s + 2 * v + 1);
         }
     }
 #pragma unroll
-    for (int j = 0; j < kSteps; ++j) {
-        const uint32_t v = j * kTileThreads + threadIdx.x;
+    for (int j = 0; j < V / 2; ++j) {
+        const uint32_t v = j * blockDim.x + threadIdx.x;
         if (v < n8) {
             uint4 o;
             o.x = pack_bf16x2(a[j].x, a[j].y);
@@ -265,7 +272,7 @@ __device__ __forceinline__ uint32_t find_tile(const TileSeg* segs, uint32_t n_se
 // Against CTAs that walk 64 KiB shares in 32 KiB rounds (us a pass, the cases
 // of the sweep above): 109.9 / 818 / 766 / 921; requests pulled between
 // stores (92 MB a launch) 54.7 -> 51.8.
-template <Mode M, int BLOB>
+template <Mode M, int V, int BLOB>
 __device__ __forceinline__ void tile_copy(const TileParams<BLOB>& p) {
     constexpr bool kToUser = M == Mode::Get;
     const TileSeg* segs = reinterpret_cast<const TileSeg*>(p.blob);
@@ -287,9 +294,9 @@ __device__ __forceinline__ void tile_copy(const TileParams<BLOB>& p) {
         asm volatile("prefetch.global.L2 [%0];" ::"l"(src + threadIdx.x * 128u));
     pdl_wait_then_release();
     if (cast)
-        tile_cast(dst, src, len);
+        tile_cast<V>(dst, src, len);
     else
-        tile_copy_bytes(dst, src, len);
+        tile_copy_bytes<V>(dst, src, len);
 }
 
 // ---------------------------------------------------------------- warp tiles
@@ -348,7 +355,7 @@ template <Mode M, int BLOB>
 __device__ __forceinline__ void warp_tile(const TileParams<BLOB>& p) {
     constexpr bool kToUser = M == Mode::Get;
     const uint32_t lane = threadIdx.x & 31u;
-    const uint32_t tile = blockIdx.x * (kWarpThreads / 32) + (threadIdx.x >> 5);
+    const uint32_t tile = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (tile >= p.h.n_tiles) {
         pdl_wait_then_release();
         return;
@@ -496,28 +503,28 @@ __device__ __forceinline__ void warp_tile(const TileParams<BLOB>& p) {
 // Entry points (one per operation and kind of tile, so that profiles name
 // them). A move's source and destination are both pool pages; as warp tiles
 // it is a put.
-template <int BLOB>
-__global__ void __launch_bounds__(kTileThreads, T2I_TUNE_TILE_BLOCKS)
+template <int V, int BLOB>
+__global__ void __launch_bounds__(kTileMaxThreads<V>, 2048 / kTileMaxThreads<V>)
     scatter_put_kernel(const __grid_constant__ TileParams<BLOB> p) {
-    tile_copy<Mode::Put, BLOB>(p);
+    tile_copy<Mode::Put, V, BLOB>(p);
 }
-template <int BLOB>
-__global__ void __launch_bounds__(kTileThreads, T2I_TUNE_TILE_BLOCKS)
+template <int V, int BLOB>
+__global__ void __launch_bounds__(kTileMaxThreads<V>, 2048 / kTileMaxThreads<V>)
     gather_get_kernel(const __grid_constant__ TileParams<BLOB> p) {
-    tile_copy<Mode::Get, BLOB>(p);
+    tile_copy<Mode::Get, V, BLOB>(p);
 }
-template <int BLOB>
-__global__ void __launch_bounds__(kTileThreads, T2I_TUNE_TILE_BLOCKS)
+template <int V, int BLOB>
+__global__ void __launch_bounds__(kTileMaxThreads<V>, 2048 / kTileMaxThreads<V>)
     compact_move_kernel(const __grid_constant__ TileParams<BLOB> p) {
-    tile_copy<Mode::Move, BLOB>(p);
+    tile_copy<Mode::Move, V, BLOB>(p);
 }
 template <int BLOB>
-__global__ void __launch_bounds__(kWarpThreads, T2I_TUNE_WARP_BLOCKS)
+__global__ void __launch_bounds__(1024, 1)
     scatter_put_warp_kernel(const __grid_constant__ TileParams<BLOB> p) {
     warp_tile<Mode::Put, BLOB>(p);
 }
 template <int BLOB>
-__global__ void __launch_bounds__(kWarpThreads, T2I_TUNE_WARP_BLOCKS)
+__global__ void __launch_bounds__(1024, 1)
     gather_get_warp_kernel(const __grid_constant__ TileParams<BLOB> p) {
     warp_tile<Mode::Get, BLOB>(p);
 }

@@ -26,24 +26,28 @@ inline bool pages_are_run(const Seg& s) {
     return true;
 }
 
-// The kernel of a mode, a kind of tile and a tier of parameters.
-template <Mode M, bool WARP, int BLOB>
+// The kernel of a mode, a kind of tile (V = 0: warp tiles, else CTA tiles of V
+// vectors per thread) and a tier of parameters.
+template <Mode M, int V, int BLOB>
 const void* tile_kernel() {
-    if constexpr (WARP)
+    if constexpr (V == 0)
         return M == Mode::Get ? reinterpret_cast<const void*>(gather_get_warp_kernel<BLOB>)
                               : reinterpret_cast<const void*>(scatter_put_warp_kernel<BLOB>);
     else
-        return M == Mode::Put   ? reinterpret_cast<const void*>(scatter_put_kernel<BLOB>)
-               : M == Mode::Get ? reinterpret_cast<const void*>(gather_get_kernel<BLOB>)
-                                : reinterpret_cast<const void*>(compact_move_kernel<BLOB>);
+        return M == Mode::Put   ? reinterpret_cast<const void*>(scatter_put_kernel<V, BLOB>)
+               : M == Mode::Get ? reinterpret_cast<const void*>(gather_get_kernel<V, BLOB>)
+                                : reinterpret_cast<const void*>(compact_move_kernel<V, BLOB>);
 }
 
 // Packs and launches the segments of one pool.
 class TileLauncher {
   public:
     // launches (nullable) counts the kernels launched
-    TileLauncher(uint64_t pool, uint32_t page_shift, uint64_t* launches)
-        : pool_(pool), page_shift_(page_shift), launches_(launches) {}
+    TileLauncher(uint64_t pool, uint32_t page_shift, int device, uint64_t* launches)
+        : pool_(pool), page_shift_(page_shift), launches_(launches) {
+        int n = 0;
+        if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, device) == cudaSuccess) sms_ = unsigned(n);
+    }
 
     // kPrefetchSources, or 0 when a source is (or may be) other than device memory
     uint32_t flags = kPrefetchSources;
@@ -62,8 +66,8 @@ class TileLauncher {
 
     uint64_t pool_;
     uint32_t page_shift_;
+    unsigned sms_ = 0;
     uint64_t* launches_;
-    std::vector<Seg> aligned_, general_;
     std::vector<uint32_t> lp_;  // page lists of the launch being packed
     alignas(16) unsigned char param_buf_[sizeof(TileParams<kBlobLarge>)];
 };
@@ -82,18 +86,29 @@ t2i_status TileLauncher::launch_one(uint32_t n_seg, uint32_t n_tiles, cudaStream
     p->h.n_tiles = n_tiles;
     p->h.flags = flags;
     std::memcpy(p->blob + n_seg * sizeof(TileSeg), lp_.data(), lp_.size() * sizeof(uint32_t));
-    constexpr uint32_t kPerCta = WARP ? kWarpThreads / 32 : 1;
+    const void* fn;
+    unsigned grid = n_tiles, threads = kTileThreads;
+    if constexpr (WARP) {
+        fn = tile_kernel<M, 0, BLOB>();
+        unsigned warps = kWarpThreads / 32;
+        if (n_tiles <= kWarpMaxPerSm * sms_) warps = (n_tiles + sms_ - 1) / sms_;
+        threads = 32 * warps;
+        grid = (n_tiles + warps - 1) / warps;
+    } else {
+        if (n_tiles <= kTileMaxPerSm * sms_) threads = kTileWaveThreads[(n_tiles + sms_ - 1) / sms_];
+        fn = threads >= 512 ? tile_kernel<M, 2, BLOB>() : tile_kernel<M, 4, BLOB>();
+    }
     void* args[] = {param_buf_};
     cudaLaunchConfig_t lc = {};
-    lc.gridDim = dim3((n_tiles + kPerCta - 1) / kPerCta);
-    lc.blockDim = dim3(WARP ? kWarpThreads : kTileThreads);
+    lc.gridDim = dim3(grid);
+    lc.blockDim = dim3(threads);
     lc.stream = stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     lc.attrs = attr;
     lc.numAttrs = 1;
-    const cudaError_t e = cudaLaunchKernelExC(&lc, tile_kernel<M, WARP, BLOB>(), args);
+    const cudaError_t e = cudaLaunchKernelExC(&lc, fn, args);
     if (e != cudaSuccess) {
         error = std::string("kernel launch failed: ") + cudaGetErrorString(e);
         return T2I_ERR_CUDA;
@@ -157,8 +172,10 @@ t2i_status TileLauncher::launch_tiles(const std::vector<Seg>& segs, cudaStream_t
     return flush();
 }
 
-// Aligned segments that fit CTA tiles run as those; the rest of the call, or
-// all of it, is one launch of warp tiles.
+// A call whose segments are all aligned and fit CTA tiles runs as those, any
+// other call as warp tiles. (A call of aligned and other segments is not
+// split: 200 ragged objects, 26 MB, took 33.7 us a put and get with their
+// aligned ones as CTA tiles, 32.4 as one launch.)
 //
 // On one stream, CTA tiles ramp up and drain fastest. Launches that overlap
 // hide each other's ramps; what counts then is bytes in flight against
@@ -169,30 +186,25 @@ t2i_status TileLauncher::launch_tiles(const std::vector<Seg>& segs, cudaStream_t
 // pages of 2 MiB 98.6 / 94.7, 127.5 / 126.3, 188.6 / 189.4; of 1 MiB 99.1 /
 // 94.8, 127.9 / 126.2, 188.9 / 189.4; of 256 KiB, scattered, 101.1 / 95.1, 130.6
 // / 126.3, 191.4 / 189.5; of 64 KiB 128.8 / 122.7, 132.4 / 126.8, 195.5 / 190.2.
-// On one stream 2 MiB pages 111.9 / 113.4 (14 MB), 195.8 / 201.5 (58 MB).
+// On one stream 2 MiB pages 70.2 / 69.5 (14 MB), 195.8 / 201.5 (58 MB).
 template <Mode M>
 t2i_status TileLauncher::launch(const std::vector<Seg>& segs, cudaStream_t stream) {
     uint64_t bytes = 0, tiles = 0;
-    uint32_t n_other = 0;
-    bool runs = true;  // every aligned segment is one page or one run of pages
+    bool aligned = true;
+    bool runs = true;  // every segment is one page or one run of pages
     for (const Seg& s : segs) {
-        if (s.user & 15u) {
-            ++n_other;
-            continue;
-        }
         const uint64_t n = s.nbytes_flags & kSegBytesMask;
         bytes += n;
         tiles += (n + kTileBytes - 1) / kTileBytes;
+        aligned = aligned && (s.user & 15u) == 0;
+        if (!aligned) break;
         if (page_shift_ < kLargePageShift && runs) runs = pages_are_run(s);
     }
     const bool near = runs || page_shift_ >= kLargePageShift;
-    const bool fit = (runs || page_shift_ >= kTileShift) && !(overlapped && !(near && bytes >= kOverlappedTileMinBytes));
-    // large enough, and the tiles filled well enough: a half-empty one costs as much as a full one
-    if (!fit || bytes < kTileMinBytes || tiles * kTileBytes > bytes + bytes / 4) return launch_tiles<M, true>(segs, stream);
-    if (n_other == 0) return launch_tiles<M, false>(segs, stream);
-    aligned_.clear();
-    general_.clear();
-    for (const Seg& s : segs) ((s.user & 15u) == 0 ? aligned_ : general_).push_back(s);
-    const t2i_status st = launch_tiles<M, false>(aligned_, stream);
-    return st != T2I_OK ? st : launch_tiles<M, true>(general_, stream);
+    // CTA tiles: each in one page or run; the call large enough; its tiles filled
+    // well enough (a half-empty one costs as much as a full one)
+    const bool fit = aligned && (runs || page_shift_ >= kTileShift) && bytes >= kTileMinBytes &&
+                     tiles * kTileBytes <= bytes + bytes / 4 &&
+                     (!overlapped || (near && bytes >= kOverlappedTileMinBytes));
+    return fit ? launch_tiles<M, false>(segs, stream) : launch_tiles<M, true>(segs, stream);
 }

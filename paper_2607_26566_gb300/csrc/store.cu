@@ -113,7 +113,7 @@ class Store {
     Store(void* pool, const t2i_store_config& cfg, int device)
         : pool_(reinterpret_cast<uint64_t>(pool)), cfg_(cfg), device_(device),
           ctl_(cfg.pool_bytes / cfg.page_bytes, cfg.page_bytes, cfg.alloc_policy),
-          launcher_(pool_, uint32_t(log2_exact(cfg.page_bytes)), &ctl_.counters().launches) {
+          launcher_(pool_, uint32_t(log2_exact(cfg.page_bytes)), device, &ctl_.counters().launches) {
         handle_.core = &ctl_;
         handle_.owned = false;
         handle_.mu = &mu;
@@ -1000,7 +1000,8 @@ template <int... BLOB>
 cudaError_t load_gathers() {
     cudaFuncAttributes a;
     cudaError_t e = cudaSuccess;
-    for (const void* fn : {tile_kernel<Mode::Get, false, BLOB>()..., tile_kernel<Mode::Get, true, BLOB>()...})
+    for (const void* fn : {tile_kernel<Mode::Get, 0, BLOB>()..., tile_kernel<Mode::Get, 2, BLOB>()...,
+                           tile_kernel<Mode::Get, 4, BLOB>()...})
         if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, fn);
     return e;
 }
@@ -1090,7 +1091,7 @@ extern "C" t2i_status t2i_gather_noalloc(const void* pool_dev, uint64_t pool_byt
         DeviceGuard g(device);
         const t2i_status st = noalloc_setup(device);
         if (st != T2I_OK) return st;
-        TileLauncher launcher(pa, uint32_t(shift), nullptr);
+        TileLauncher launcher(pa, uint32_t(shift), device, nullptr);
         const std::vector<Seg> segs{{da, nbytes | (cast ? kCastFlag : 0), pages, n_pages}};
         const t2i_status ls = launcher.launch<Mode::Get>(segs, static_cast<cudaStream_t>(cuda_stream));
         if (ls != T2I_OK) set_thread_error("t2i_gather_noalloc: " + launcher.error);
