@@ -133,6 +133,7 @@ t2i_status TileLauncher::launch_tiles(const std::vector<Seg>& segs, cudaStream_t
                               : bytes <= size_t(kBlobTiny)  ? launch_one<M, WARP, kBlobTiny>(n_seg, tiles, stream)
                               : bytes <= size_t(kBlobSmall) ? launch_one<M, WARP, kBlobSmall>(n_seg, tiles, stream)
                               : bytes <= size_t(kBlobMid)   ? launch_one<M, WARP, kBlobMid>(n_seg, tiles, stream)
+                              : bytes <= size_t(kBlobHalf)  ? launch_one<M, WARP, kBlobHalf>(n_seg, tiles, stream)
                                                             : launch_one<M, WARP, kBlobLarge>(n_seg, tiles, stream);
         n_seg = tiles = 0;
         lp_.clear();

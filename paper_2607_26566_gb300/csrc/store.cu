@@ -1012,7 +1012,7 @@ bool g_noalloc_loaded[kNoAllocMaxDevices];
 t2i_status noalloc_setup(int device) {
     std::lock_guard<std::mutex> lock(g_noalloc_mu);
     if (g_noalloc_loaded[device]) return T2I_OK;
-    const cudaError_t e = load_gathers<kBlobTiny, kBlobSmall, kBlobMid, kBlobLarge>();
+    const cudaError_t e = load_gathers<kBlobTiny, kBlobSmall, kBlobMid, kBlobHalf, kBlobLarge>();
     if (e != cudaSuccess) {
         set_thread_error(std::string("t2i_gather_noalloc: cannot load the kernels: ") + cudaGetErrorString(e));
         return T2I_ERR_CUDA;
