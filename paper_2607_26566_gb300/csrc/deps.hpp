@@ -64,8 +64,15 @@ class StreamDeps {
     // not be called; the marks are kept for streams to come.
     bool several() const { return streams_.size() > 1; }
 
+    // Whether the current call and those before it came on several streams in
+    // turn (a change of stream within the last kInterleave calls), so that
+    // their work is likely to overlap. A hint for the shape of a launch only.
+    static constexpr uint32_t kInterleave = 16;
+    bool interleaved() const { return since_change_ < kInterleave; }
+
     // --- one call on stream index `si`
     void begin(int si) {
+        since_change_ = si != cur_ ? 0 : since_change_ < kInterleave ? since_change_ + 1 : kInterleave;
         cur_ = si;
         need_.assign(streams_.size(), 0);
         wait_all_ = false;
@@ -179,6 +186,7 @@ class StreamDeps {
     std::vector<PageDeps> pages_;
     std::vector<uint32_t> need_;
     int cur_ = 0;
+    uint32_t since_change_ = kInterleave;  // calls since the last change of stream
     bool wait_all_ = false;
 };
 

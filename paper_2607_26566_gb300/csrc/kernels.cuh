@@ -59,7 +59,10 @@ constexpr int kBlobLarge = 31 * 1024;  // header + blob stays below the 32,764-b
 // 128 x 4 93.9 / 815 / 760 / 904. Without the L2 prefetch: 102.0 / 811 / 757 / 902.
 constexpr uint32_t kTileShift = 14;
 constexpr uint32_t kTileBytes = 1u << kTileShift;
-constexpr unsigned kTileThreads = 512;
+#ifndef T2I_TUNE_TILE_THREADS
+#define T2I_TUNE_TILE_THREADS 512
+#endif
+constexpr unsigned kTileThreads = T2I_TUNE_TILE_THREADS;
 #ifndef T2I_TUNE_TILE_MIN_BYTES
 #define T2I_TUNE_TILE_MIN_BYTES (4ull << 20)
 #endif
@@ -74,6 +77,15 @@ constexpr unsigned kTileThreads = 512;
 #endif
 constexpr unsigned kTileWaveThreads[] = {1024, 1024, 1024, 672, 512, 384, 320, 288, 256};
 constexpr unsigned kTileMaxPerSm = T2I_TUNE_TILE_BALANCE ? 8 : 0;
+// Threads of a launch beside other streams' launches. Those hide each other's
+// ramps; what counts then is bytes in flight against latency (longer in
+// scattered pages), and six CTAs an SM hold 96 KiB, the four of 512 threads 64.
+// In 512 / 384 / 320 / 256 threads on four streams: handoffs of 58 MB a call in
+// scattered 64 KiB pages 195.5 / 191.0 / 190.0 / 190.3 us a pass, of 29 MB 132.4
+// / 128.6 / 127.0 / 126.9, of 14 MB in 2 MiB pages 98.6 / 96.7 / 94.9 / 94.8, of
+// 92 MB 814.8 / 813.7 / 813.7 / 814.9; adapter gets of 98 MB 6.83 / 7.06 / 7.11 /
+// 7.14 TB/s; pulls of 92 MB 7.06 / 7.15 / 7.16 / 7.15.
+constexpr unsigned kTileOverlapThreads = 320;
 // vectors per thread V: T x V >= 1,024 vectors a tile
 template <int V>
 constexpr unsigned kTileMaxThreads = V == 2 ? 1024 : 384;
@@ -117,14 +129,36 @@ struct TileHeader {
     uint32_t n_seg;
     uint32_t page_shift;
     uint32_t n_tiles;
-    uint32_t flags;  // kPrefetchSources, or 0
+    uint32_t flags;  // kPrefetchSources, kTileTable
+    uint32_t table_at;     // byte offset of the segment table in blob (kTileTable)
+    uint32_t table_shift;  // tiles per entry, as a power of two
 };
-static_assert(sizeof(TileHeader) == 24, "TileHeader layout");
+static_assert(sizeof(TileHeader) == 32, "TileHeader layout");
+// The launch carries a table of segments: uint16 entry e is the segment of tile
+// e << table_shift, so a tile's segment lies between two entries. Searching
+// 256 descriptors takes 8 dependent loads of parameters, which miss the
+// constant cache in turn; with the table it takes one or two. A 40 MB get of
+// 256 adapter tensors took 12.2 us without it and 11.8 with it, such gets on
+// four streams ran at 6.13 TB/s and 6.90. The table costs the host about a
+// nanosecond a segment, so it comes with segments of many tiles only; and a
+// long launch alone on the GPU gains nothing from CTAs that start sooner (a
+// 2.7 GB get took 753 us without and 757 with it, compaction of 1 GiB in calls
+// of up to 512 MiB 891 and 899), so it has none.
+constexpr uint32_t kTileTable = 2u;
+#ifndef T2I_TUNE_TABLE_MIN_SEGS
+#define T2I_TUNE_TABLE_MIN_SEGS 5
+#endif
+constexpr uint32_t kTableMinSegs = T2I_TUNE_TABLE_MIN_SEGS;
+constexpr uint32_t kTableMinTilesPerSeg = 8;
+#ifndef T2I_TUNE_TABLE_MAX_BYTES
+#define T2I_TUNE_TABLE_MAX_BYTES (256u << 20)
+#endif
+constexpr uint32_t kTableMaxBytes = T2I_TUNE_TABLE_MAX_BYTES;
 
 template <int BLOB>
 struct TileParams {
     TileHeader h;
-    alignas(8) unsigned char blob[BLOB];  // TileSeg[n_seg], then uint32 pages[]
+    alignas(8) unsigned char blob[BLOB];  // TileSeg[n_seg], then uint32 pages[], then the uint16 table
 };
 
 enum class Mode { Put, Get, Move };
@@ -250,8 +284,15 @@ __device__ __forceinline__ void pdl_wait_then_release() {
 }
 
 // The last segment that starts at or before this tile.
-__device__ __forceinline__ uint32_t find_tile(const TileSeg* segs, uint32_t n_seg, uint32_t tile) {
-    uint32_t lo = 0, hi = n_seg - 1;
+template <int BLOB>
+__device__ __forceinline__ uint32_t find_tile(const TileParams<BLOB>& p, uint32_t tile) {
+    const TileSeg* segs = reinterpret_cast<const TileSeg*>(p.blob);
+    uint32_t lo = 0, hi = p.h.n_seg - 1;
+    if (p.h.flags & kTileTable) {
+        const uint16_t* table = reinterpret_cast<const uint16_t*>(p.blob + p.h.table_at) + (tile >> p.h.table_shift);
+        lo = table[0];
+        hi = table[1];
+    }
     while (lo < hi) {
         const uint32_t mid = (lo + hi + 1) >> 1;
         if (segs[mid].tile0 <= tile)
@@ -278,7 +319,7 @@ template <Mode M, int V, int BLOB>
 __device__ __forceinline__ void tile_copy(const TileParams<BLOB>& p) {
     constexpr bool kToUser = M == Mode::Get;
     const TileSeg* segs = reinterpret_cast<const TileSeg*>(p.blob);
-    const uint32_t lo = find_tile(segs, p.h.n_seg, blockIdx.x);
+    const uint32_t lo = find_tile(p, blockIdx.x);
     const uint32_t off = (blockIdx.x - segs[lo].tile0) << kTileShift;
     const uint32_t len = umin(kTileBytes, segs[lo].nbytes - off);
     const uint32_t flags = segs[lo].flags;
@@ -363,7 +404,7 @@ __device__ __forceinline__ void warp_tile(const TileParams<BLOB>& p) {
         return;
     }
     const TileSeg* segs = reinterpret_cast<const TileSeg*>(p.blob);
-    const TileSeg& s = segs[find_tile(segs, p.h.n_seg, tile)];
+    const TileSeg& s = segs[find_tile(p, tile)];
     const uint32_t* pages = reinterpret_cast<const uint32_t*>(segs + p.h.n_seg);
     unsigned char* pool = reinterpret_cast<unsigned char*>(p.h.pool);
     unsigned char* user = reinterpret_cast<unsigned char*>(s.user);

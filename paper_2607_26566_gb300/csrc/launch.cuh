@@ -16,9 +16,6 @@ struct Seg {
 };
 constexpr uint64_t kCastFlag = uint64_t(1) << 63;
 constexpr uint64_t kSegBytesMask = ~kCastFlag;
-// see TileLauncher::launch
-constexpr uint32_t kLargePageShift = 20;
-constexpr uint64_t kOverlappedTileMinBytes = 48ull << 20;
 
 inline bool pages_are_run(const Seg& s) {
     for (uint32_t k = 1; k < s.n_pages; ++k)
@@ -61,6 +58,7 @@ class TileLauncher {
   private:
     template <Mode M, bool WARP>
     t2i_status launch_tiles(const std::vector<Seg>& segs, cudaStream_t stream);
+    void add_table(TileHeader* h, unsigned char* blob, size_t blob_bytes);
     template <Mode M, bool WARP, int BLOB>
     t2i_status launch_one(uint32_t n_seg, uint32_t n_tiles, cudaStream_t stream);
 
@@ -86,6 +84,9 @@ t2i_status TileLauncher::launch_one(uint32_t n_seg, uint32_t n_tiles, cudaStream
     p->h.n_tiles = n_tiles;
     p->h.flags = flags;
     std::memcpy(p->blob + n_seg * sizeof(TileSeg), lp_.data(), lp_.size() * sizeof(uint32_t));
+    if (n_seg >= kTableMinSegs && n_tiles / n_seg >= kTableMinTilesPerSeg &&
+        (overlapped || n_tiles < kTableMaxBytes / (WARP ? kWarpTileBytes : kTileBytes)))
+        add_table(&p->h, p->blob, BLOB);
     const void* fn;
     unsigned grid = n_tiles, threads = kTileThreads;
     if constexpr (WARP) {
@@ -95,7 +96,10 @@ t2i_status TileLauncher::launch_one(uint32_t n_seg, uint32_t n_tiles, cudaStream
         threads = 32 * warps;
         grid = (n_tiles + warps - 1) / warps;
     } else {
-        if (n_tiles <= kTileMaxPerSm * sms_) threads = kTileWaveThreads[(n_tiles + sms_ - 1) / sms_];
+        if (overlapped)
+            threads = kTileOverlapThreads;
+        else if (n_tiles <= kTileMaxPerSm * sms_)
+            threads = kTileWaveThreads[(n_tiles + sms_ - 1) / sms_];
         fn = threads >= 512 ? tile_kernel<M, 2, BLOB>() : tile_kernel<M, 4, BLOB>();
     }
     void* args[] = {param_buf_};
@@ -115,6 +119,27 @@ t2i_status TileLauncher::launch_one(uint32_t n_seg, uint32_t n_tiles, cudaStream
     }
     if (launches_) ++*launches_;
     return T2I_OK;
+}
+
+// Puts the segment table behind the page lists, with up to two entries a
+// segment, as far as the tier has room (it is not worth a larger tier).
+inline void TileLauncher::add_table(TileHeader* h, unsigned char* blob, size_t blob_bytes) {
+    const TileSeg* segs = reinterpret_cast<const TileSeg*>(blob);
+    const size_t at = h->n_seg * sizeof(TileSeg) + lp_.size() * sizeof(uint32_t);
+    const size_t room = std::min<size_t>(2 * h->n_seg, (blob_bytes - at) / sizeof(uint16_t));
+    if (room < 3) return;
+    uint32_t shift = 0;  // entries 0 .. ((n_tiles - 1) >> shift) + 1
+    while (((h->n_tiles - 1) >> shift) + 2 > room) ++shift;
+    const uint32_t n = ((h->n_tiles - 1) >> shift) + 2;
+    uint16_t* table = reinterpret_cast<uint16_t*>(blob + at);
+    uint32_t e = 0;
+    for (uint32_t i = 0; i < h->n_seg; ++i) {
+        const uint64_t end = i + 1 < h->n_seg ? segs[i + 1].tile0 : uint64_t(n) << shift;
+        for (; e < n && (uint64_t(e) << shift) < end; ++e) table[e] = static_cast<uint16_t>(i);
+    }
+    h->table_at = static_cast<uint32_t>(at);
+    h->table_shift = shift;
+    h->flags |= kTileTable;
 }
 
 // The segments as tiles, in as few launches as their descriptors allow.
@@ -177,17 +202,6 @@ t2i_status TileLauncher::launch_tiles(const std::vector<Seg>& segs, cudaStream_t
 // other call as warp tiles. (A call of aligned and other segments is not
 // split: 200 ragged objects, 26 MB, took 33.7 us a put and get with their
 // aligned ones as CTA tiles, 32.4 as one launch.)
-//
-// On one stream, CTA tiles ramp up and drain fastest. Launches that overlap
-// hide each other's ramps; what counts then is bytes in flight against
-// latency, and an SM holds 128 KiB of warp tiles but 64 KiB of CTA tiles. So
-// overlapped launches run as warp tiles, except large ones in large pages (or
-// runs), where latency is lowest and CTA tiles use HBM best. Handoffs of 14,
-// 29 and 58 MB a call on four streams, us a pass in CTA tiles / warp tiles:
-// pages of 2 MiB 98.6 / 94.7, 127.5 / 126.3, 188.6 / 189.4; of 1 MiB 99.1 /
-// 94.8, 127.9 / 126.2, 188.9 / 189.4; of 256 KiB, scattered, 101.1 / 95.1, 130.6
-// / 126.3, 191.4 / 189.5; of 64 KiB 128.8 / 122.7, 132.4 / 126.8, 195.5 / 190.2.
-// On one stream 2 MiB pages 70.2 / 69.5 (14 MB), 195.8 / 201.5 (58 MB).
 template <Mode M>
 t2i_status TileLauncher::launch(const std::vector<Seg>& segs, cudaStream_t stream) {
     uint64_t bytes = 0, tiles = 0;
@@ -199,13 +213,11 @@ t2i_status TileLauncher::launch(const std::vector<Seg>& segs, cudaStream_t strea
         tiles += (n + kTileBytes - 1) / kTileBytes;
         aligned = aligned && (s.user & 15u) == 0;
         if (!aligned) break;
-        if (page_shift_ < kLargePageShift && runs) runs = pages_are_run(s);
+        if (page_shift_ < kTileShift && runs) runs = pages_are_run(s);
     }
-    const bool near = runs || page_shift_ >= kLargePageShift;
     // CTA tiles: each in one page or run; the call large enough; its tiles filled
     // well enough (a half-empty one costs as much as a full one)
     const bool fit = aligned && (runs || page_shift_ >= kTileShift) && bytes >= kTileMinBytes &&
-                     tiles * kTileBytes <= bytes + bytes / 4 &&
-                     (!overlapped || (near && bytes >= kOverlappedTileMinBytes));
+                     tiles * kTileBytes <= bytes + bytes / 4;
     return fit ? launch_tiles<M, false>(segs, stream) : launch_tiles<M, true>(segs, stream);
 }

@@ -162,7 +162,7 @@ class Store {
     // ---- launches of segs_
     template <Mode M>
     t2i_status launch_segments(cudaStream_t stream) {
-        launcher_.overlapped = deps_.several();
+        launcher_.overlapped = deps_.interleaved();
         const t2i_status st = launcher_.launch<M>(segs_, stream);
         if (st != T2I_OK) err_ = launcher_.error;
         return st;

@@ -130,25 +130,48 @@ def test_gather_without_a_store_overlapping_and_captured():
         assert torch.equal(out_a, want ^ 255) and torch.equal(out_b, want)
 
 
-@pytest.mark.parametrize("P", [65536, 1 << 20])
-@pytest.mark.parametrize("n", [(48 << 20) - 16, (48 << 20) + 20])
-def test_large_calls_of_a_store_used_on_two_streams(P, n):
-    """Calls on both sides of the line between warp and CTA tiles that a store
-    used on several streams has, in scattered pages below and at the page size
-    where it lies: copy and cast, byte for byte."""
+@pytest.mark.parametrize("P", [16384, 65536, 1 << 20])
+@pytest.mark.parametrize("n", [(4 << 20) - 16, (4 << 20) + 20, (48 << 20) + 4])
+def test_large_calls_on_two_streams_in_turn(P, n):
+    """Calls whose launches are shaped to run beside other streams' (and the
+    first, which is not), on both sides of the line between warp and CTA tiles,
+    in scattered pages: copy and cast, byte for byte."""
     n_pages = -(-n // P)
     st = Store(torch.zeros(2 * n_pages * P, dtype=torch.uint8, device=DEV), P)
     scatter(st, 2 * n_pages, P, 7)
     f = torch.randn(n // 4, device=DEV)
     outs = [torch.zeros(n, dtype=torch.uint8, device=DEV), torch.zeros(n // 2, dtype=torch.uint8, device=DEV)]
     torch.cuda.synchronize()
-    for s in (torch.cuda.Stream(), torch.cuda.Stream()):
+    for s in 2 * (torch.cuda.Stream(), torch.cuda.Stream()):
         st_, ids = st.put_batch(put_descs([f]), stream=s)
         assert st_ == 0
         assert st.get_batch(get_descs([ids[0], ids[0]], outs, cast=[0, 1]), stream=s)[0] == 0
         torch.cuda.synchronize()
         assert torch.equal(outs[0], f.view(torch.uint8))
         assert torch.equal(outs[1].view(torch.bfloat16), f.to(torch.bfloat16))
+        assert st.free(ids) == 0
         outs[0].zero_()
         outs[1].zero_()
         torch.cuda.synchronize()
+
+
+@pytest.mark.parametrize("n_obj", [4, 5, 6, 300])
+def test_launches_with_a_segment_table(n_obj):
+    """Objects of many tiles, as many as bring a table of segments with the
+    launch and one fewer: sizes from one tile to a hundred, so that entries of
+    the table cover several segments and part of one; put and get (copy)."""
+    P = 65536
+    rng = np.random.default_rng(n_obj)
+    sizes = np.exp(rng.uniform(np.log(16384), np.log(100 * 16384), n_obj)).astype(np.int64) & ~15
+    sizes[0] += max(0, (5 << 20) - int(sizes.sum()))
+    offs = np.concatenate([[0], np.cumsum(sizes)])
+    n_pages = int(sum(-(-n // P) for n in sizes)) + 5
+    st = Store(torch.zeros(n_pages * P, dtype=torch.uint8, device=DEV), P)
+    scatter(st, n_pages, P, 9)
+    src = torch.randint(0, 256, (int(offs[-1]),), dtype=torch.uint8, device=DEV)
+    s, ids = st.put_batch(put_descs(src.data_ptr() + offs[:-1], nbytes=sizes))
+    assert s == 0, st.last_error()
+    out = torch.zeros_like(src)
+    assert st.get_batch(get_descs(ids, out.data_ptr() + offs[:-1], dst_bytes=sizes))[0] == 0
+    torch.cuda.synchronize()
+    assert torch.equal(out, src)
