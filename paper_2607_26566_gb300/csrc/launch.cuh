@@ -36,6 +36,32 @@ const void* tile_kernel() {
                                 : reinterpret_cast<const void*>(compact_move_kernel<V, BLOB>);
 }
 
+// Loads every kernel on the current device, once per device (the driver loads
+// a kernel, allocating device memory for it, when it is first named): calls
+// then allocate nothing and can be captured.
+template <int... BLOB>
+cudaError_t load_tier_kernels() {
+    const void* fns[] = {tile_kernel<Mode::Get, 0, BLOB>()...,  tile_kernel<Mode::Put, 0, BLOB>()...,
+                         tile_kernel<Mode::Get, 2, BLOB>()...,  tile_kernel<Mode::Get, 4, BLOB>()...,
+                         tile_kernel<Mode::Put, 2, BLOB>()...,  tile_kernel<Mode::Put, 4, BLOB>()...,
+                         tile_kernel<Mode::Move, 2, BLOB>()..., tile_kernel<Mode::Move, 4, BLOB>()...};
+    cudaFuncAttributes a;
+    cudaError_t e = cudaSuccess;
+    for (const void* fn : fns)
+        if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, fn);
+    return e;
+}
+inline cudaError_t load_kernels(int device) {
+    static std::mutex mu;
+    static std::vector<bool> loaded;
+    std::lock_guard<std::mutex> lock(mu);
+    if (loaded.size() <= size_t(device)) loaded.resize(size_t(device) + 1, false);
+    if (loaded[device]) return cudaSuccess;
+    const cudaError_t e = load_tier_kernels<kBlobTiny, kBlobSmall, kBlobMid, kBlobHalf, kBlobLarge>();
+    if (e == cudaSuccess) loaded[device] = true;
+    return e;
+}
+
 // Packs and launches the segments of one pool.
 class TileLauncher {
   public:

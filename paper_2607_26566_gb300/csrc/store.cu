@@ -833,6 +833,12 @@ t2i_status t2i_store_create(void* pool_dev, const t2i_store_config* cfg, int dev
     }
     Store* s = nullptr;
     try {
+        t2i::DeviceGuard g(device);
+        const cudaError_t e = t2i::load_kernels(device);
+        if (e != cudaSuccess) {
+            t2i::set_thread_error(std::string("t2i_store_create: cannot load the kernels: ") + cudaGetErrorString(e));
+            return T2I_ERR_CUDA;
+        }
         s = new Store(pool_dev, *cfg, device);
     } catch (const std::exception& e) {
         t2i::set_thread_error(std::string("t2i_store_create: host error: ") + e.what());
@@ -993,34 +999,7 @@ uint64_t noalloc_pages_per_launch(uint64_t page_bytes) {
     return std::min<uint64_t>(kNoAllocMaxPagesPerLaunch, std::max<uint64_t>(1, (uint64_t(1) << 36) / page_bytes));
 }
 
-// Loads every gather kernel on the current device (the driver loads a kernel,
-// allocating device memory for it, when it is first named), once per device:
-// later calls then allocate nothing and can be captured.
-template <int... BLOB>
-cudaError_t load_gathers() {
-    cudaFuncAttributes a;
-    cudaError_t e = cudaSuccess;
-    for (const void* fn : {tile_kernel<Mode::Get, 0, BLOB>()..., tile_kernel<Mode::Get, 2, BLOB>()...,
-                           tile_kernel<Mode::Get, 4, BLOB>()...})
-        if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, fn);
-    return e;
-}
 constexpr int kNoAllocMaxDevices = 64;
-std::mutex g_noalloc_mu;
-bool g_noalloc_loaded[kNoAllocMaxDevices];
-
-t2i_status noalloc_setup(int device) {
-    std::lock_guard<std::mutex> lock(g_noalloc_mu);
-    if (g_noalloc_loaded[device]) return T2I_OK;
-    const cudaError_t e = load_gathers<kBlobTiny, kBlobSmall, kBlobMid, kBlobHalf, kBlobLarge>();
-    if (e != cudaSuccess) {
-        set_thread_error(std::string("t2i_gather_noalloc: cannot load the kernels: ") + cudaGetErrorString(e));
-        return T2I_ERR_CUDA;
-    }
-    g_noalloc_loaded[device] = true;
-    return T2I_OK;
-}
-
 }  // namespace
 }  // namespace t2i
 
@@ -1089,8 +1068,11 @@ extern "C" t2i_status t2i_gather_noalloc(const void* pool_dev, uint64_t pool_byt
             return T2I_ERR_INVALID;
         }
         DeviceGuard g(device);
-        const t2i_status st = noalloc_setup(device);
-        if (st != T2I_OK) return st;
+        const cudaError_t e = load_kernels(device);
+        if (e != cudaSuccess) {
+            set_thread_error(std::string("t2i_gather_noalloc: cannot load the kernels: ") + cudaGetErrorString(e));
+            return T2I_ERR_CUDA;
+        }
         TileLauncher launcher(pa, uint32_t(shift), device, nullptr);
         const std::vector<Seg> segs{{da, nbytes | (cast ? kCastFlag : 0), pages, n_pages}};
         const t2i_status ls = launcher.launch<Mode::Get>(segs, static_cast<cudaStream_t>(cuda_stream));

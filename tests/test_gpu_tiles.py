@@ -175,3 +175,29 @@ def test_launches_with_a_segment_table(n_obj):
     assert st.get_batch(get_descs(ids, out.data_ptr() + offs[:-1], dst_bytes=sizes))[0] == 0
     torch.cuda.synchronize()
     assert torch.equal(out, src)
+
+
+@pytest.mark.parametrize("tiles_per_sm", [1, 4, 5, 8, 9, 17, 31, 32, 33])
+@pytest.mark.parametrize("mis", [0, 2])
+def test_one_wave_launches(tiles_per_sm, mis):
+    """Launches sized around the whole numbers of tiles an SM can hold at once
+    (the CTA's threads follow from them, up to 1,024), aligned and not: a put
+    and a get with the cast of one fp32 object."""
+    sms = torch.cuda.get_device_properties(DEV).multi_processor_count
+    tile = 4096 if mis else TILE
+    n = (tiles_per_sm if mis else min(tiles_per_sm, 9)) * sms * tile - 4 * (tiles_per_sm % 3)
+    P = 2 << 20
+    st = Store(torch.zeros((n // P + 2) * P, dtype=torch.uint8, device=DEV), P)
+    f = torch.randn(n // 4, device=DEV)
+    src = torch.zeros(n + 16, dtype=torch.uint8, device=DEV)
+    src[mis:mis + n] = f.view(torch.uint8)
+    s, ids = st.put_batch(put_descs([src.data_ptr() + mis], nbytes=[n]))
+    assert s == 0, st.last_error()
+    out, bf = torch.zeros(n + 16, dtype=torch.uint8, device=DEV), torch.zeros(n // 2 + 16, dtype=torch.uint8, device=DEV)
+    assert st.get_batch(get_descs(ids, [out.data_ptr() + mis], dst_bytes=[n]))[0] == 0
+    assert st.get_batch(get_descs(ids, [bf.data_ptr() + mis], dst_bytes=[n // 2], cast=1))[0] == 0
+    torch.cuda.synchronize()
+    assert torch.equal(out[mis:mis + n], f.view(torch.uint8))
+    assert torch.equal(bf[mis:mis + n // 2].view(torch.bfloat16), f.to(torch.bfloat16))
+    for o, m in ((out, n), (bf, n // 2)):
+        assert not o[:mis].any() and not o[mis + m:].any()
