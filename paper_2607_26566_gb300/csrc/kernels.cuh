@@ -389,11 +389,13 @@ __device__ __forceinline__ void store_shifted(uint4* d, const uint4 (&r)[V], uin
 // a CTA's share, and a call with any mix of alignments is one launch instead
 // of two. Bound by HBM in large ones, which come here for their alignment or
 // their small pages. Before (CTAs walking shares, pieces realigned in shared
-// memory) and after: 646 tensors of 256 B to 36 KiB got in 30.8 -> 25.3 us, 40
-// ragged objects put and got in 18.5 -> 15.9; 1 GiB puts from unaligned
-// sources 7.13 -> 7.21 TB/s, gets into unaligned destinations 7.08 -> 7.13,
-// casts into 2-byte aligned ones 6.92 -> 7.18; 64 MiB in scattered 8 KiB pages
-// put 4.97 -> 7.25, got 4.81 -> 6.50, cast 3.24 -> 6.53.
+// memory) and after, kernel times of one launch on an idle GPU: 646 tensors of
+// 256 B to 36 KiB got in 10.6 -> 5.0 us, 40 ragged objects put in 14.5 (two
+// launches) -> 4.9, got in 10.4 -> 4.9; 1 GiB puts from unaligned sources 7.13
+// -> 7.21 TB/s, gets into unaligned destinations 7.08 -> 7.13, casts into 2-byte
+// aligned ones 6.92 -> 7.18; 64 MiB in scattered 8 KiB pages put 4.97 -> 7.25,
+// got 4.81 -> 6.50, cast 3.24 -> 6.53. Tiles of 1 or 2 KiB in small launches
+// (fewer vectors a lane, more warps) changed no pass.
 template <Mode M, int BLOB>
 __device__ __forceinline__ void warp_tile(const TileParams<BLOB>& p) {
     constexpr bool kToUser = M == Mode::Get;

@@ -175,6 +175,7 @@ inline void TileLauncher::add_table(TileHeader* h, unsigned char* blob, size_t b
 template <Mode M, bool WARP>
 t2i_status TileLauncher::launch_tiles(const std::vector<Seg>& segs, cudaStream_t stream) {
     constexpr uint64_t kTile = WARP ? kWarpTileBytes : kTileBytes;
+    static_assert(offsetof(TileParams<kBlobLarge>, blob) == sizeof(TileHeader), "the same place in every tier");
     TileSeg* const out = reinterpret_cast<TileSeg*>(param_buf_ + sizeof(TileHeader));
     uint32_t n_seg = 0, tiles = 0;
     lp_.clear();
