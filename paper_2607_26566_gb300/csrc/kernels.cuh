@@ -86,6 +86,11 @@ constexpr unsigned kTileMaxPerSm = T2I_TUNE_TILE_BALANCE ? 8 : 0;
 // 92 MB 814.8 / 813.7 / 813.7 / 814.9; adapter gets of 98 MB 6.83 / 7.06 / 7.11 /
 // 7.14 TB/s; pulls of 92 MB 7.06 / 7.15 / 7.16 / 7.15.
 constexpr unsigned kTileOverlapThreads = 320;
+// Such launches of fewer bytes run as warp tiles: of 11.5 MB on four streams,
+// issued from C, 6.82 TB/s, against 6.85 / 6.70 / 6.66 / 6.55 in CTA tiles of 512
+// / 384 / 320 / 256 threads; of 14 MB 94.7 us a pass against 98.6 / 96.7 / 94.9 /
+// 94.8. At 29 MB both kinds run alike.
+constexpr uint64_t kTileOverlapMinBytes = 20ull << 20;
 // vectors per thread V: T x V >= 1,024 vectors a tile
 template <int V>
 constexpr unsigned kTileMaxThreads = V == 2 ? 1024 : 384;

@@ -244,7 +244,8 @@ t2i_status TileLauncher::launch(const std::vector<Seg>& segs, cudaStream_t strea
     }
     // CTA tiles: each in one page or run; the call large enough; its tiles filled
     // well enough (a half-empty one costs as much as a full one)
-    const bool fit = aligned && (runs || page_shift_ >= kTileShift) && bytes >= kTileMinBytes &&
+    const bool fit = aligned && (runs || page_shift_ >= kTileShift) &&
+                     bytes >= (overlapped ? kTileOverlapMinBytes : kTileMinBytes) &&
                      tiles * kTileBytes <= bytes + bytes / 4;
     return fit ? launch_tiles<M, false>(segs, stream) : launch_tiles<M, true>(segs, stream);
 }
