@@ -10,17 +10,22 @@
 // One object (or page) of a batch, on its way to a launch.
 struct Seg {
     uint64_t user;          // device-visible address of the user's side
-    uint64_t nbytes_flags;  // bytes in the pool, kCastFlag
+    uint64_t nbytes_flags;  // bytes in the pool, kCastFlag (and kRunFlag, set by the launcher)
     const uint32_t* pages;
     uint32_t n_pages;
 };
 constexpr uint64_t kCastFlag = uint64_t(1) << 63;
-constexpr uint64_t kSegBytesMask = ~kCastFlag;
+constexpr uint64_t kRunFlag = uint64_t(1) << 62;  // one page, or consecutive ones
+constexpr uint64_t kSegBytesMask = ~(kCastFlag | kRunFlag);
 
+// Whether the pages are consecutive. Scattered pages mostly show at the last
+// one; a run is then read in one pass without branches.
 inline bool pages_are_run(const Seg& s) {
-    for (uint32_t k = 1; k < s.n_pages; ++k)
-        if (s.pages[k] != s.pages[0] + k) return false;
-    return true;
+    const uint32_t first = s.pages[0], n = s.n_pages;
+    if (s.pages[n - 1] != first + (n - 1)) return false;
+    uint32_t off = 0;
+    for (uint32_t k = 0; k < n; ++k) off |= s.pages[k] ^ (first + k);
+    return off == 0;
 }
 
 // The kernel of a mode, a kind of tile (V = 0: warp tiles, else CTA tiles of V
@@ -79,7 +84,7 @@ class TileLauncher {
     std::string error;
 
     template <Mode M>
-    t2i_status launch(const std::vector<Seg>& segs, cudaStream_t stream);
+    t2i_status launch(std::vector<Seg>& segs, cudaStream_t stream);
 
   private:
     template <Mode M, bool WARP>
@@ -197,7 +202,7 @@ t2i_status TileLauncher::launch_tiles(const std::vector<Seg>& segs, cudaStream_t
     for (const Seg& s : segs) {
         const uint64_t nbytes = s.nbytes_flags & kSegBytesMask;
         const uint32_t cast = (s.nbytes_flags & kCastFlag) != 0;
-        const bool run = pages_are_run(s);
+        const bool run = (s.nbytes_flags & kRunFlag) != 0;
         const uint64_t step = run ? seg_pages : list_pages;
         for (uint64_t p0 = 0; p0 < s.n_pages; p0 += step) {
             const uint64_t np = std::min<uint64_t>(step, s.n_pages - p0);
@@ -230,17 +235,18 @@ t2i_status TileLauncher::launch_tiles(const std::vector<Seg>& segs, cudaStream_t
 // split: 200 ragged objects, 26 MB, took 33.7 us a put and get with their
 // aligned ones as CTA tiles, 32.4 as one launch.)
 template <Mode M>
-t2i_status TileLauncher::launch(const std::vector<Seg>& segs, cudaStream_t stream) {
+t2i_status TileLauncher::launch(std::vector<Seg>& segs, cudaStream_t stream) {
     uint64_t bytes = 0, tiles = 0;
     bool aligned = true;
     bool runs = true;  // every segment is one page or one run of pages
-    for (const Seg& s : segs) {
+    for (Seg& s : segs) {
         const uint64_t n = s.nbytes_flags & kSegBytesMask;
         bytes += n;
         tiles += (n + kTileBytes - 1) / kTileBytes;
         aligned = aligned && (s.user & 15u) == 0;
-        if (!aligned) break;
-        if (page_shift_ < kTileShift && runs) runs = pages_are_run(s);
+        const bool run = s.n_pages == 1 || pages_are_run(s);
+        if (run) s.nbytes_flags |= kRunFlag;
+        runs = runs && run;
     }
     // CTA tiles: each in one page or run; the call large enough; its tiles filled
     // well enough (a half-empty one costs as much as a full one)

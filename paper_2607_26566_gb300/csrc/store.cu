@@ -1074,7 +1074,7 @@ extern "C" t2i_status t2i_gather_noalloc(const void* pool_dev, uint64_t pool_byt
             return T2I_ERR_CUDA;
         }
         TileLauncher launcher(pa, uint32_t(shift), device, nullptr);
-        const std::vector<Seg> segs{{da, nbytes | (cast ? kCastFlag : 0), pages, n_pages}};
+        std::vector<Seg> segs{{da, nbytes | (cast ? kCastFlag : 0), pages, n_pages}};
         const t2i_status ls = launcher.launch<Mode::Get>(segs, static_cast<cudaStream_t>(cuda_stream));
         if (ls != T2I_OK) set_thread_error("t2i_gather_noalloc: " + launcher.error);
         return ls;
