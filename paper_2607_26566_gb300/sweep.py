@@ -6,7 +6,7 @@ is timed by ``bench.py --lib`` in the same process order, alternating, for a
 few repetitions, and one table line per run shows the figures the choices in
 the kernels' comments were made on.
 
-    python -m paper_2607_26566_gb300.sweep base= pf24=T2I_TUNE_PREFETCH_BYTES=24576 \\
+    python -m paper_2607_26566_gb300.sweep base= nopf=T2I_TUNE_PREFETCH=0 \\
         --bench "--no-e2e --no-cpu --rows adapters --adapter-calls 2000 --steps 30" --reps 2
 
 A variant is ``NAME=DEF[,DEF...]`` (``NAME=`` alone: the defaults). Builds go
