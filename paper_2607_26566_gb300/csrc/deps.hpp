@@ -33,7 +33,7 @@ class StreamDeps {
     struct PageDeps {
         Dep writer;
         Dep readers[2];
-        uint8_t more_readers = 0;  // > 2 reading streams since the last write
+        uint8_t more_readers = 0;  // > 2 reading streams since the last write (2: a view may be among the others)
     };
     static constexpr uint32_t kRing = 64;
     // a reader whose reads are not calls of the store (a view): later
@@ -75,7 +75,7 @@ class StreamDeps {
         since_change_ = si != cur_ ? 0 : since_change_ < kInterleave ? since_change_ + 1 : kInterleave;
         cur_ = si;
         need_.assign(streams_.size(), 0);
-        wait_all_ = false;
+        wait_all_ = 0;
     }
     void reads(uint32_t page) { note(pages_[page].writer); }
     void writes(uint32_t page) {
@@ -83,13 +83,15 @@ class StreamDeps {
         note(d.writer);
         note(d.readers[0]);
         note(d.readers[1]);
-        if (d.more_readers) wait_all_ = true;
+        if (wait_all_ < d.more_readers) wait_all_ = d.more_readers;
     }
     // Makes the call's stream wait for what it depends on.
     cudaError_t wait() {
         cudaStream_t s = streams_[cur_].s;
         for (size_t j = 0; j < streams_.size(); ++j) {
-            const uint32_t q = wait_all_ ? streams_[j].seq : need_[j];
+            uint32_t q = need_[j];
+            if (wait_all_ && q < streams_[j].seq) q = streams_[j].seq;
+            if (wait_all_ == 2 && streams_[j].viewed) q = kOpen;
             if (int(j) == cur_ || q == 0) continue;
             cudaError_t e = wait_for(static_cast<int>(j), q, s);
             if (e != cudaSuccess) return e;
@@ -120,13 +122,17 @@ class StreamDeps {
     void mark_read(uint32_t page, uint32_t seq) {
         PageDeps& d = pages_[page];
         const Dep me{seq, static_cast<uint16_t>(cur_)};
+        if (seq == kOpen) streams_[cur_].viewed = true;
         for (Dep& r : d.readers) {
             if (r.seq == 0 || r.stream == me.stream) {
-                r = me;
+                // a view lasts until the page is written: the stream's later
+                // calls do not end its reads
+                if (r.seq != kOpen) r = me;
                 return;
             }
         }
-        d.more_readers = 1;
+        const uint8_t more = seq == kOpen ? 2 : 1;
+        if (d.more_readers < more) d.more_readers = more;
     }
 
     // Waits on the host for everything every known stream has been given.
@@ -156,6 +162,7 @@ class StreamDeps {
         uint32_t ring_seq[kRing] = {};  // the call each ring event was last recorded for
         cudaEvent_t lazy = nullptr; // "everything so far" on this stream
         uint32_t lazy_seq = 0;
+        bool viewed = false;        // a view was given to it: reads beyond its calls
     };
 
     static cudaError_t ensure(cudaEvent_t* e) {
@@ -187,7 +194,7 @@ class StreamDeps {
     std::vector<uint32_t> need_;
     int cur_ = 0;
     uint32_t since_change_ = kInterleave;  // calls since the last change of stream
-    bool wait_all_ = false;
+    uint8_t wait_all_ = 0;  // the call overwrites a page with more_readers
 };
 
 }  // namespace t2i

@@ -717,6 +717,36 @@ def test_view_is_ordered_after_its_writer_and_before_reuse():
     assert torch.equal(z, x)
 
 
+@pytest.mark.parametrize("others", ["get on the view's stream", "two more views", "gets on three streams"])
+def test_view_lasts_until_its_pages_are_reused(others):
+    """Calls made after a view, on its stream or on others, do not end its
+    reads: a put that reuses the pages still waits for a late read in place."""
+    P = 64 * 1024
+    st = make_store(8 * P, P, alloc_policy=1)
+    s1, s2, s3, s4, s5 = (torch.cuda.Stream() for _ in range(5))
+    x = torch.randint(0, 256, (8 * P,), dtype=torch.uint8, device=DEV)
+    y = torch.randint(0, 256, (8 * P,), dtype=torch.uint8, device=DEV)
+    outs = [torch.zeros_like(x) for _ in range(3)]
+    s, (ix,) = st.put_batch(put_descs([x]))
+    assert s == 0
+    torch.cuda.synchronize()
+    gets = {"get on the view's stream": (s5, s1), "two more views": (), "gets on three streams": (s2, s3, s4)}[others]
+    viewers = (s1, s2, s3) if others == "two more views" else (s1,)
+    views = [st.tensor_view(int(ix), stream=v)[1] for v in viewers]
+    for g, o in zip(gets, outs):
+        assert st.get_batch(get_descs([int(ix)], [o]), stream=g)[0] == 0
+    copies = []
+    for v, t in zip(viewers, views):
+        _late(v, 30)
+        with torch.cuda.stream(v):
+            copies.append(t.clone())
+    assert st.free([int(ix)]) == 0
+    s, (iy,) = st.put_batch(put_descs([y]), stream=s5)   # the same pages
+    assert s == 0 and st.ctl.object(int(iy))[2] == list(range(8))
+    torch.cuda.synchronize()
+    assert all(torch.equal(c, x) for c in copies) and all(torch.equal(o, x) for _, o in zip(gets, outs))
+
+
 def test_pull_between_stores_vs_oracle():
     """A consumer's store pulls objects from a producer's store page to page
     (§5.2): statuses, ids, placement and bytes as the oracle's pull."""
