@@ -138,7 +138,7 @@ class StreamDeps {
     // Waits on the host for everything every known stream has been given.
     void synchronize_all() {
         for (State& st : streams_) {
-            if (st.seq == 0) continue;
+            if (st.seq == 0 && !st.viewed) continue;
             if (ensure(&st.lazy) == cudaSuccess && cudaEventRecord(st.lazy, st.s) == cudaSuccess)
                 cudaEventSynchronize(st.lazy);
         }

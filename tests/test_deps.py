@@ -31,8 +31,8 @@ inline cudaError_t cudaEventSynchronize(cudaEvent_t e) { if (e->s) host_seen[e->
 """
 
 # Commands: "<verb><stream>", verbs v(iew), g(et), p(ut) of page 0 and k: work
-# the caller gives the stream itself. Output: the work of A, B and C that the
-# last command's stream has waited for.
+# the caller gives the stream itself; x: the store is destroyed. Output: the
+# work of A, B and C that the last command's stream (x: the host) has waited for.
 DRIVER = r"""
 #include <cstdio>
 #include <string>
@@ -53,6 +53,11 @@ int main(int argc, char** argv) {
     };
     for (int i = 1; i < argc; ++i) {
         const char verb = argv[i][0];
+        if (verb == 'x') {
+            d.synchronize_all();
+            for (int k = 0; k < 3; ++k) std::printf("%d ", host_seen[&s[k]]);
+            return 0;
+        }
         FakeStream* st = &s[argv[i][1] - 'A'];
         if (verb == 'k') st->work++;
         else call(verb, st);
@@ -94,3 +99,8 @@ def test_a_put_waits_for_the_readers_of_the_pages_it_reuses(driver, calls, want)
     if calls.split()[-1] == "pB":
         got[1] = 0  # its own stream
     assert got == want
+
+
+@pytest.mark.parametrize("calls,want", [("gA kA gB x", [2, 1, 0]), ("vA kA x", [1, 0, 0]), ("gA vB kB x", [1, 1, 0])])
+def test_destroy_waits_for_every_stream(driver, calls, want):
+    assert waited(driver, calls) == want
