@@ -351,8 +351,9 @@ t2i_status t2i_inject_launch_failure(t2i_store* store, uint32_t countdown);
  * device memory: no cudaMalloc, no cudaFree, no library routine that
  * allocates.
  *
- * pool_dev, pool_bytes: the pool, device memory of `device`; pool_bytes is a
- *   positive multiple of page_bytes, a power of two in [256 B, 1 GiB].
+ * pool_dev, pool_bytes: the pool, device memory of `device`, 16-byte aligned
+ *   (its pages are read in 16-byte vectors); pool_bytes is a positive multiple
+ *   of page_bytes, a power of two in [256 B, 1 GiB].
  * pages, n_pages: the object's page list in byte order (a host array of
  *   page indices into the pool, e.g. from t2i_ctl_object), read during the
  *   call. n_pages = ceil(nbytes / page_bytes), at most 64 times

@@ -1030,6 +1030,10 @@ extern "C" t2i_status t2i_gather_noalloc(const void* pool_dev, uint64_t pool_byt
             return T2I_ERR_INVALID;
         }
         if (nbytes == 0) return T2I_OK;
+        if (reinterpret_cast<uint64_t>(pool_dev) & 15u) {
+            set_thread_error("t2i_gather_noalloc: the pool must be 16-byte aligned");
+            return T2I_ERR_INVALID;
+        }
         if (!pages || !dst_dev) {
             set_thread_error("t2i_gather_noalloc: null page list or destination");
             return T2I_ERR_INVALID;
