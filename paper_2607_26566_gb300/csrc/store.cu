@@ -1034,6 +1034,10 @@ extern "C" t2i_status t2i_gather_noalloc(const void* pool_dev, uint64_t pool_byt
             set_thread_error("t2i_gather_noalloc: the pool must be 16-byte aligned");
             return T2I_ERR_INVALID;
         }
+        if (reinterpret_cast<uint64_t>(pool_dev) + pool_bytes < pool_bytes) {
+            set_thread_error("t2i_gather_noalloc: the pool's range wraps around");
+            return T2I_ERR_INVALID;
+        }
         if (!pages || !dst_dev) {
             set_thread_error("t2i_gather_noalloc: null page list or destination");
             return T2I_ERR_INVALID;

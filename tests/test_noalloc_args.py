@@ -19,3 +19,9 @@ def refused(lib, why, pool=1 << 40, pool_bytes=16 * P, page=0, dst=1 << 41):
 def test_a_pool_that_is_not_16_byte_aligned(lib, off):
     """The kernels read pages as 16-byte vectors."""
     assert refused(lib, b"16-byte aligned", pool=(1 << 40) + off)
+
+
+@pytest.mark.parametrize("pool_bytes,page", [((1 << 64) - P, 16), ((1 << 64) - (1 << 40), 1 << 20), ((1 << 64) - (1 << 30), 0)])
+def test_a_pool_that_wraps_around_the_address_space(lib, pool_bytes, page):
+    """Its end lies below its start, so it would pass as part of its allocation."""
+    assert refused(lib, b"wraps", pool_bytes=pool_bytes, page=page)
