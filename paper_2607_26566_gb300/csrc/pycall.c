@@ -10,9 +10,9 @@
  * METH_FASTCALL, and keeps the interpreter lock for the call: a few
  * microseconds of host work, unless the call waits for the store's own lock
  * (another thread is inside the store) or for room in a full launch queue,
- * during which other Python threads wait too (the ctypes binding releases
- * the lock instead). Marshalling only: every check, page table step and
- * byte move happens in the library.
+ * during which other Python threads wait too (the ctypes binding, and
+ * free_ids, release the lock instead). Marshalling only: every check, page
+ * table step and byte move happens in the library.
  */
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
@@ -129,14 +129,20 @@ static PyObject* py_get_batch_for(PyObject* self, PyObject* const* args, Py_ssiz
 }
 
 /* free_ids(store, ids) -> status, or None if ids is not a one-dimensional
- * uint64 array: t2i_free of every id in it. */
+ * uint64 array: t2i_free of every id in it. Other Python threads run
+ * meanwhile: the call may wait for a thread that is inside the store, and
+ * that one (in the ctypes binding) for a launch queue that only a Python
+ * callback empties. */
 static PyObject* py_free_ids(PyObject* self, PyObject* const* args, Py_ssize_t n) {
     void* h;
     Py_buffer view;
     (void)self;
     if (!nargs_ok(n, 2, "free_ids") || !arg_ptr(args, 0, &h)) return NULL;
     if (!ids_of(args[1], -1, &view)) Py_RETURN_NONE;
-    const t2i_status st = t2i_free((t2i_store*)h, (const t2i_id*)view.buf, (uint32_t)view.shape[0]);
+    t2i_status st;
+    Py_BEGIN_ALLOW_THREADS
+    st = t2i_free((t2i_store*)h, (const t2i_id*)view.buf, (uint32_t)view.shape[0]);
+    Py_END_ALLOW_THREADS
     PyBuffer_Release(&view);
     return PyLong_FromLong(st);
 }
