@@ -55,7 +55,7 @@ static int ids_of(PyObject* obj, Py_ssize_t n, Py_buffer* view) {
     }
     const char* f = view->format;
     if (view->itemsize == 8 && f && (f[0] == 'L' || f[0] == 'Q') && f[1] == '\0' && view->ndim >= 1 &&
-        (n < 0 ? view->ndim == 1 && view->shape[0] <= 0xFFFFFFFF : view->shape[0] >= n))
+        (n < 0 ? view->ndim == 1 && view->shape[0] <= 0xFFFFFFFF : view->shape[0] >= n && view->len / 8 >= n))
         return 1;
     PyBuffer_Release(view);
     return 0;

@@ -288,9 +288,14 @@ class Store:
         if self._fast is not None:
             if ids is None:
                 return self._fast.get_batch(self._hi, p.addr, p.n, p.out_addr, _stream(stream))
-            st = self._fast.get_batch_for(self._hi, p.addr, p.n, ids, p.out_addr, _stream(stream))
-            if st is not None:
-                return st
+            if isinstance(ids, np.ndarray):
+                s = _stream(stream)
+                st = self._fast.get_batch_for(self._hi, p.addr, p.n, ids, p.out_addr, s)
+                if st is not None:
+                    return st
+                # an array whose buffer does not say plain uint64 (it is not aligned)
+                if ids.dtype == np.uint64 and ids.flags.c_contiguous and len(ids) >= p.n and ids.size >= p.n:
+                    return self._fast.get_batch_ids(self._hi, p.addr, p.n, ids.ctypes.data, p.out_addr, s)
         if ids is not None:
             p.descs["id"] = ids
         return self._lib.t2i_get_batch(self._h, p.addr, p.n, p.out_addr, _stream(stream))
