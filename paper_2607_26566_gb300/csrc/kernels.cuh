@@ -51,12 +51,13 @@ constexpr int kBlobHalf = 16384;
 constexpr int kBlobLarge = 31 * 1024;  // header + blob stays below the 32,764-byte parameter limit
 
 // ---- tiled launches (see tile_copy): the segments cut into 16 KiB tiles,
-// one CTA each. 512 threads x 2 vectors, from a sweep on GB300 (us a pass;
-// put + get of B=4 requests of 45 MB on one stream / of 16 B=8 requests of
-// 92 MB on four / get of 2.7 GB / put, compaction and get of 1 GiB): 512 x 2
-// 94.1 / 810 / 755 / 895; 1024 x 2 94.6 / 810 / 765 / 901; 512 x 4 98.2 / 814 /
-// 759 / 904; 256 x 4 96.7 / 815 / 760 / 904; 256 x 2 95.1 / 812 / 757 / 900;
-// 128 x 4 93.9 / 815 / 760 / 904. Without the L2 prefetch: 102.0 / 811 / 757 / 902.
+// one CTA each. 512 threads x 2 vectors, from a sweep on GB300 over threads x
+// vectors (us a pass; put + get of B=4 requests of 45 MB on one stream / of 16
+// B=8 requests of 92 MB on four / get of 2.7 GB / put, compaction and get of
+// 1 GiB). Tiles of 16 KiB: 512 x 2 94.1 / 810 / 755 / 895; 256 x 4 96.7 / 815 /
+// 760 / 904. Of 32 KiB: 1024 x 2 94.6 / 810 / 765 / 901; 512 x 4 98.2 / 814 / 759 /
+// 904. Of 8 KiB: 256 x 2 95.1 / 812 / 757 / 900; 128 x 4 93.9 / 815 / 760 / 904.
+// 512 x 2 without the L2 prefetch: 102.0 / 811 / 757 / 902.
 constexpr uint32_t kTileShift = 14;
 constexpr uint32_t kTileBytes = 1u << kTileShift;
 #ifndef T2I_TUNE_TILE_THREADS
@@ -71,7 +72,8 @@ constexpr unsigned kTileThreads = T2I_TUNE_TILE_THREADS;
 // spare, the next grid's CTAs fill some SMs early and others late, and its
 // slowest SM decides: eight B=1 requests on one stream (11.5 MB, 705 tiles a
 // call) took 62.4 us a pass in 512 threads, 58.0 in 384; of 14 MB (870) 74.7,
-// 70.0 in 320; a launch of over 8 tiles an SM takes 512.
+// 70.0 in 320; a launch of over 8 tiles an SM takes 512. (kTileMinBytes makes
+// two tiles an SM or more on 152 SMs: the first two entries serve larger chips.)
 #ifndef T2I_TUNE_TILE_BALANCE
 #define T2I_TUNE_TILE_BALANCE 1
 #endif
@@ -91,9 +93,24 @@ constexpr unsigned kTileOverlapThreads = 320;
 // / 384 / 320 / 256 threads; of 14 MB 94.7 us a pass against 98.6 / 96.7 / 94.9 /
 // 94.8. At 29 MB both kinds run alike.
 constexpr uint64_t kTileOverlapMinBytes = 20ull << 20;
-// vectors per thread V: T x V >= 1,024 vectors a tile
+// Vectors per thread, and the most threads of a kernel of V vectors.
+constexpr int tile_vec(unsigned threads) { return threads >= 512 ? 2 : 4; }
 template <int V>
 constexpr unsigned kTileMaxThreads = V == 2 ? 1024 : 384;
+// A CTA's threads copy a whole tile in one round, within their kernel's bound.
+constexpr bool tile_threads_ok(unsigned threads) {
+    const int v = tile_vec(threads);
+    return threads % 32 == 0 && threads * unsigned(v) * 16 >= kTileBytes &&
+           threads <= (v == 2 ? kTileMaxThreads<2> : kTileMaxThreads<4>);
+}
+constexpr bool tile_wave_threads_ok() {
+    for (unsigned t : kTileWaveThreads)
+        if (!tile_threads_ok(t)) return false;
+    return kTileMaxPerSm < sizeof(kTileWaveThreads) / sizeof(kTileWaveThreads[0]);
+}
+static_assert(tile_threads_ok(kTileThreads), "T2I_TUNE_TILE_THREADS does not cover a tile");
+static_assert(tile_threads_ok(kTileOverlapThreads), "kTileOverlapThreads does not cover a tile");
+static_assert(tile_wave_threads_ok(), "kTileWaveThreads: an entry does not cover a tile, or one is missing");
 // Aligned launches of at least this many bytes run as CTA tiles, others as
 // warp tiles. On one stream eight B=1 requests took (us a pass) 47.1 in CTA
 // tiles and 59.7 in warp tiles at 7 MB a call, 58.0 and 59.3 at 11.5 MB, four

@@ -131,7 +131,7 @@ t2i_status TileLauncher::launch_one(uint32_t n_seg, uint32_t n_tiles, cudaStream
             threads = kTileOverlapThreads;
         else if (n_tiles <= kTileMaxPerSm * sms_)
             threads = kTileWaveThreads[(n_tiles + sms_ - 1) / sms_];
-        fn = threads >= 512 ? tile_kernel<M, 2, BLOB>() : tile_kernel<M, 4, BLOB>();
+        fn = tile_vec(threads) == 2 ? tile_kernel<M, 2, BLOB>() : tile_kernel<M, 4, BLOB>();
     }
     void* args[] = {param_buf_};
     cudaLaunchConfig_t lc = {};
