@@ -201,6 +201,7 @@ class Store {
 #define T2I_TUNE_COMPACT_FIRST 64
 #endif
     static constexpr size_t kCompactFirstBatch = T2I_TUNE_COMPACT_FIRST;  // moves in the first launch
+    static_assert(kCompactFirstBatch >= 1, "a compaction plans its moves batch by batch");
     static_assert(kMovesPerLaunch * sizeof(TileSeg) <= size_t(kBlobLarge), "moves per launch");
 };
 
