@@ -606,7 +606,7 @@ def time_tiny(device, reps: int = 20):
 
 
 def time_unaligned(device, reps: int = 10, nbytes: int = 1 << 30):
-    """The any-alignment kernels on one 1 GiB object (2 MiB pages, a 2 GiB
+    """Any alignment: the warp-tile kernels on one 1 GiB object (2 MiB pages, a 2 GiB
     pool): puts from sources 1, 4 and 8 bytes past a 16-byte boundary, gets
     into destinations 1 and 3 bytes past one, fp32 -> bf16 casts into
     destinations 2 and 6 bytes past one, each beside its aligned form. Every

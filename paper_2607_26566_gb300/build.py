@@ -72,7 +72,7 @@ def is_stale() -> bool:
 def build(verbose: bool = False, ptxas_info: bool = False, defines=(), out: str | None = None,
           build_dir: str | None = None) -> str:
     """Compiles and links the library; returns its path. Raises on failure.
-    ``defines`` (e.g. ["T2I_TUNE_VEC=8"]) and ``out`` build a variant of the
+    ``defines`` (e.g. ["T2I_TUNE_PREFETCH=0"]) and ``out`` build a variant of the
     kernels' launch shape elsewhere (tuning sweeps)."""
     lib_path = out or LIB
     bdir = build_dir or BUILD

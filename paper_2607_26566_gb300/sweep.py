@@ -1,7 +1,7 @@
 """Tuning sweeps of the kernels' compile-time launch shapes (GPU).
 
 Each variant is the library built with some ``T2I_TUNE_*`` definitions
-(``csrc/kernels.cuh``, ``csrc/launch.cuh``, ``csrc/store.cu``); every variant
+(``csrc/kernels.cuh``, ``csrc/store.cu``); every variant
 is timed by ``bench.py --lib`` in the same process order, alternating, for a
 few repetitions, and one table line per run shows the figures the choices in
 the kernels' comments were made on.

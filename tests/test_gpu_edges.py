@@ -105,7 +105,7 @@ def test_empty_and_zero_byte_batches():
 
 def test_unaligned_cast_and_copy_kernels():
     """Sources at every 16-byte misalignment (put), destinations at every
-    misalignment (copy) and every even one (cast): the any-alignment kernels."""
+    misalignment (copy) and every even one (cast)."""
     P = 8192
     st = store(512 * P, P)
     rng = np.random.default_rng(2)
@@ -161,9 +161,9 @@ def test_cast_into_two_byte_aligned_destinations():
 
 
 def test_object_larger_than_64_gib():
-    """An object of 65 GiB + a ragged tail in 1 GiB pages: its launch byte
-    space is split into segments of at most 64 GiB, so 32-bit granule
-    offsets never wrap. Every GiB of the get is compared with the put."""
+    """An object of 65 GiB + a ragged tail in 1 GiB pages: split into segments
+    of at most 1 GiB, so that 32-bit offsets in one never wrap. Every GiB of
+    the get is compared with the put."""
     G = 1 << 30
     if torch.cuda.get_device_properties(0).total_memory < 180 * G:
         pytest.skip("needs a GPU with room for two 66 GiB buffers")
@@ -187,14 +187,13 @@ def test_object_larger_than_64_gib():
     del x
 
 
-def test_large_unaligned_launches_take_chunks():
-    """A 704 MiB object put from a source 3 bytes past alignment and got into
-    destinations 5 bytes (copy) and 2 bytes (cast) past it: launches large
-    enough for chunks from the work counter (at least 1 MiB per resident
-    CTA of the any-alignment kernels, 4 per SM), in those kernels."""
-    P = 2 << 20
-    n = 704 << 20
-    st = store(360 * P, P)
+@pytest.mark.parametrize("P", [64 << 10, 2 << 20])
+def test_unaligned_object_over_1_gib(P):
+    """An object a little over 1 GiB in consecutive pages, put from a source 3
+    bytes past alignment and got into destinations 5 bytes (copy) and 2 bytes
+    (cast) past it: one run of pages, split into two segments at 1 GiB."""
+    n = (1 << 30) + 3 * P + 20
+    st = store((n // P + 2) * P, P)
     g = torch.Generator(device=DEV)
     g.manual_seed(400)
     f = torch.randn(n // 4, generator=g, device=DEV)
@@ -214,10 +213,9 @@ def test_large_unaligned_launches_take_chunks():
 
 @pytest.mark.parametrize("P", [256, 1024, 4096, 16384])
 def test_small_page_rounds(P):
-    """Objects spanning many pages smaller than a copy round: rounds that
-    cover several pages in put, get, get with a cast in the same launch, and
-    the any-alignment kernels (a source 3 bytes past alignment); every byte
-    against the oracle's get."""
+    """Objects spanning many pages, smaller than a warp tile and larger: put
+    (one source 3 bytes past alignment), get, and a get with a cast in the
+    same launch; every byte against the oracle's get."""
     rng = np.random.default_rng(P)
     n_pages = (6 << 20) // P
     st = store(n_pages * P, P)

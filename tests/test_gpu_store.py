@@ -799,12 +799,10 @@ def test_pull_waits_for_a_late_producer():
     assert torch.equal(out, x)
 
 
-def test_chunked_launches_on_eight_streams_at_once():
-    """Large gets (>= 1 MiB per CTA: chunks from the work counters) on eight
-    streams at once, each stream with its own counter; every byte checked,
-    twice in a row (each launch leaves its counter at zero)."""
+def test_large_gets_on_eight_streams_at_once():
+    """Large gets on eight streams at once, twice in a row; every byte checked."""
     P = 2 << 20
-    n = 600 << 20                                    # 300 pages, 1.3 MiB per CTA of the get grid
+    n = 600 << 20                                    # 300 pages
     st = make_store(8 * (n // P) * P + 8 * P, P)
     streams = [torch.cuda.Stream() for _ in range(8)]
     xs = [torch.randint(0, 256, (n,), dtype=torch.uint8, device=DEV) for _ in range(8)]
@@ -821,9 +819,8 @@ def test_chunked_launches_on_eight_streams_at_once():
             assert torch.equal(x, o)
 
 
-def test_streams_beyond_the_counter_slots_split_statically():
-    """A store has work counters for its first 64 streams; later streams use
-    equal static shares. A large get on the 70th stream is still exact."""
+def test_a_store_used_on_seventy_streams():
+    """Small gets on 70 streams, then a large one on the last of them."""
     P = 2 << 20
     n = 600 << 20
     st = make_store(n + 8 * P, P)

@@ -178,15 +178,18 @@ def test_launches_with_a_segment_table(n_obj):
     assert torch.equal(out, src)
 
 
-@pytest.mark.parametrize("tiles_per_sm", [1, 4, 5, 8, 9, 17, 31, 32, 33])
-@pytest.mark.parametrize("mis", [0, 2])
-def test_one_wave_launches(tiles_per_sm, mis):
-    """Launches sized around the whole numbers of tiles an SM can hold at once
-    (the CTA's threads follow from them, up to 1,024), aligned and not: a put
-    and a get with the cast of one fp32 object."""
+@pytest.mark.parametrize("extra", [-1, 0, 1])
+@pytest.mark.parametrize("mis,tiles_per_sm", [(0, k) for k in range(2, 10)]
+                         + [(2, k) for k in (1, 4, 5, 8, 9, 17, 31, 32, 33)])
+def test_one_wave_launches(mis, tiles_per_sm, extra):
+    """Launches of a whole number of tiles for every SM, one more and one fewer
+    (the CTA's threads follow from it): aligned (CTA tiles: 1,024 threads for two
+    an SM down to 256 for eight, more than one wave for nine) and not (warp
+    tiles, one CTA an SM up to 32 warps): a put, a get and a get with the cast
+    of one fp32 object."""
     sms = torch.cuda.get_device_properties(DEV).multi_processor_count
     tile = 4096 if mis else TILE
-    n = (tiles_per_sm if mis else min(tiles_per_sm, 9)) * sms * tile - 4 * (tiles_per_sm % 3)
+    n = (tiles_per_sm * sms + extra) * tile - 4 * (tiles_per_sm % 3)
     P = 2 << 20
     st = Store(torch.zeros((n // P + 2) * P, dtype=torch.uint8, device=DEV), P)
     f = torch.randn(n // 4, device=DEV)

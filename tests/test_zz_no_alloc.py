@@ -6,9 +6,8 @@ or PyTorch's caching allocator has already reserved.
 Every output is compared with what the oracle fixes for it: the object's own
 bytes (get(put(x)) == x), or, with the cast, the oracle's round-to-nearest-
 even of those bytes (oracle.cast, written independently of the kernels).
-Each case makes two calls in a row, because every call shares the library's
-static scratch counters and the second must not see what the first left
-behind. The cast inputs are random bit patterns, so NaNs, infinities,
+Each case makes two calls in a row: the second must not see what the first
+left behind. The cast inputs are random bit patterns, so NaNs, infinities,
 subnormals and exact ties all occur.
 
 This file is collected last on purpose: a failure here stops a first-failure
@@ -43,10 +42,14 @@ def noalloc(pool, P, pages, nbytes, dst_addr, dst_bytes, cast, stream=None):
                                   len(pg), nbytes, dst_addr, dst_bytes, cast, 0, s.cuda_stream)
 
 
-def stored(P, pool_pages, x):
-    """A store holding x; returns (store, pool, id, page list)."""
+def stored(P, pool_pages, x, scattered=False):
+    """A store holding x, in pages in order or scattered over the pool;
+    returns (store, pool, id, page list)."""
     pool = torch.empty(pool_pages * P, dtype=torch.uint8, device=DEV)
     st = Store(pool, P)
+    if scattered:
+        s, one = st.put_batch(put_descs(np.zeros(pool_pages, np.uint64), nbytes=np.full(pool_pages, P)))
+        assert s == 0 and st.free(np.random.default_rng(P).permutation(one)) == 0
     s, (i,) = st.put_batch(put_descs([x]))
     assert s == 0, st.last_error()
     return st, pool, int(i), st.ctl.object(int(i))[2]
@@ -99,11 +102,11 @@ def test_two_calls_match_the_oracle(cast):
 
 
 def test_two_calls_multi_launch_unaligned():
-    """9,000 pages of 256 B (two launches, two scratch counters) copied into a
-    destination 3 bytes past 16-byte alignment (the any-alignment copy)."""
+    """9,000 scattered pages of 256 B (two launches) copied into a destination
+    3 bytes past 16-byte alignment."""
     P = 256
     x = torch.randint(0, 256, (9000 * P - 100,), dtype=torch.uint8, device=DEV)
-    st, pool, oid, pages = stored(P, 9500, x)
+    st, pool, oid, pages = stored(P, 9500, x, scattered=True)
     assert len(pages) == 9000
     want = expected(x, 0)
     for out in run_twice(pool, P, pages, x, 0, 3):
@@ -112,12 +115,12 @@ def test_two_calls_multi_launch_unaligned():
 
 @pytest.mark.parametrize("offset", [2, 6, 14])
 def test_cast_into_2_byte_aligned_destination_two_launches(offset):
-    """An fp32 object of 9,000 pages of 256 B with a ragged last page (two
-    launches) cast into a destination that is 2-byte but not 16-byte
-    aligned (the any-alignment cast)."""
+    """An fp32 object of 9,000 scattered pages of 256 B with a ragged last page
+    (two launches), cast into a destination that is 2-byte but not 16-byte
+    aligned."""
     P = 256
     x = random_f32_bits((9000 * P - 100) // 4, seed=10 + offset)
-    st, pool, oid, pages = stored(P, 9500, x)
+    st, pool, oid, pages = stored(P, 9500, x, scattered=True)
     assert len(pages) == 9000
     want = expected(x, 1)
     for out in run_twice(pool, P, pages, x, 1, offset):
@@ -126,8 +129,8 @@ def test_cast_into_2_byte_aligned_destination_two_launches(offset):
 
 @pytest.mark.parametrize("offset", [0, 6])
 def test_two_calls_large_object_cast(offset):
-    """256 MiB of fp32 in 2 MiB pages (~18 chunks per CTA), cast to bf16
-    into an aligned destination and one 6 bytes past alignment."""
+    """256 MiB of fp32 in 2 MiB pages, cast to bf16 into an aligned destination
+    and one 6 bytes past alignment."""
     P = 2 << 20
     x = random_f32_bits(64 << 20, seed=20 + offset)
     st, pool, oid, pages = stored(P, 130, x)
@@ -137,8 +140,8 @@ def test_two_calls_large_object_cast(offset):
 
 
 def test_sizes_beyond_the_maximum_are_rejected():
-    """More pages than 64 launches of scratch counters cover, a page list
-    that does not match nbytes, and a page outside the pool: INVALID with a
+    """More pages than 64 launches of scattered pages hold, a page list that
+    does not match nbytes, and a page outside the pool: INVALID with a
     message, nothing enqueued."""
     P = 256
     pool = torch.empty(1 << 20, dtype=torch.uint8, device=DEV)
