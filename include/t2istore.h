@@ -156,7 +156,8 @@ typedef struct t2i_object_info {
  * `device`. pool_dev must be device memory of that device, 256-byte aligned.
  * The store never frees pool_dev and allocates no device memory of its own.
  * Errors: INVALID (geometry, pointer), CUDA (device query failed, or the
- * kernels could not be loaded). On error *out is NULL and t2i_last_error(NULL) describes it.     */
+ * kernels could not be loaded). On error *out is NULL and
+ * t2i_last_error(NULL) describes it.                                        */
 t2i_status t2i_store_create(void* pool_dev, const t2i_store_config* cfg, int device, t2i_store** out);
 
 /* Frees the store's host state and events after waiting for

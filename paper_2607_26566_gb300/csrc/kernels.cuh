@@ -417,11 +417,12 @@ __device__ __forceinline__ void store_shifted(uint4* d, const uint4 (&r)[V], uin
 // their small pages. Before (CTAs walking shares, pieces realigned in shared
 // memory) and after, kernel times of one launch on an idle GPU: 646 tensors of
 // 256 B to 36 KiB got in 10.6 -> 5.0 us, 40 ragged objects put in 14.5 (two
-// launches) -> 4.9, got in 10.4 -> 4.9; 1 GiB puts from unaligned sources 7.13
-// -> 7.21 TB/s, gets into unaligned destinations 7.08 -> 7.13, casts into 2-byte
-// aligned ones 6.92 -> 7.18; 64 MiB in scattered 8 KiB pages put 4.97 -> 7.25,
-// got 4.81 -> 6.50, cast 3.24 -> 6.53. Tiles of 1 or 2 KiB in small launches
-// (fewer vectors a lane, more warps) changed no pass.
+// launches) -> 4.9, got in 10.4 -> 4.9. Ten launches back to back: 1 GiB puts from
+// unaligned sources 7.13 -> 7.21 TB/s, gets into unaligned destinations 7.08 ->
+// 7.13, casts into 2-byte aligned ones 6.92 -> 7.18 (timed alone, such a put
+// 331 -> 327 us, a get 329 -> 322); 64 MiB in scattered 8 KiB pages put
+// 4.97 -> 7.25, got 4.81 -> 6.50, cast 3.24 -> 6.53. Tiles of 1 or 2 KiB in small
+// launches (fewer vectors a lane, more warps) changed no pass.
 template <Mode M, int BLOB>
 __device__ __forceinline__ void warp_tile(const TileParams<BLOB>& p) {
     constexpr bool kToUser = M == Mode::Get;

@@ -993,13 +993,14 @@ const char* t2i_last_error(const t2i_store* store) {
 // The paper has no counterpart.
 namespace t2i {
 namespace {
+// The most pages of a call, as the header gives it: as many as 64 launches of
+// scattered pages carry, and at most 64 times 64 GiB. (The kernels have no such
+// bound: it stands because callers may count on the refusal.)
 constexpr uint64_t kNoAllocMaxLaunches = 64;
 constexpr uint64_t kNoAllocMaxPagesPerLaunch = (kBlobLarge - sizeof(TileSeg)) / sizeof(uint32_t);
-// the most pages of a call: 64 launches of scattered pages, at most 64 GiB each
 uint64_t noalloc_pages_per_launch(uint64_t page_bytes) {
     return std::min<uint64_t>(kNoAllocMaxPagesPerLaunch, std::max<uint64_t>(1, (uint64_t(1) << 36) / page_bytes));
 }
-
 constexpr int kNoAllocMaxDevices = 64;
 }  // namespace
 }  // namespace t2i
