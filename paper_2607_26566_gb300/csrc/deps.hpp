@@ -121,18 +121,30 @@ class StreamDeps {
     }
     void mark_read(uint32_t page, uint32_t seq) {
         PageDeps& d = pages_[page];
-        const Dep me{seq, static_cast<uint16_t>(cur_)};
-        if (seq == kOpen) streams_[cur_].viewed = true;
         for (Dep& r : d.readers) {
-            if (r.seq == 0 || r.stream == me.stream) {
+            if (r.seq == 0) {
+                r = {seq, static_cast<uint16_t>(cur_)};
+                return;
+            }
+            if (r.stream == cur_) {
                 // a view lasts until the page is written: the stream's later
                 // calls do not end its reads
-                if (r.seq != kOpen) r = me;
+                if (r.seq != kOpen) r.seq = seq;
                 return;
             }
         }
-        const uint8_t more = seq == kOpen ? 2 : 1;
-        if (d.more_readers < more) d.more_readers = more;
+        if (d.more_readers == 0) d.more_readers = 1;
+    }
+    void mark_view(uint32_t page) {
+        PageDeps& d = pages_[page];
+        streams_[cur_].viewed = true;
+        for (Dep& r : d.readers) {
+            if (r.seq == 0 || r.stream == cur_) {
+                r = {kOpen, static_cast<uint16_t>(cur_)};
+                return;
+            }
+        }
+        d.more_readers = 2;
     }
 
     // Waits on the host for everything every known stream has been given.

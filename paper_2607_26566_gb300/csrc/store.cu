@@ -538,7 +538,7 @@ t2i_status Store::view(t2i_id id, cudaStream_t stream, void** ptr, uint64_t* nby
     for (uint32_t pg : o->pages) deps_.reads(pg);
     cudaError_t we = deps_.wait();
     if (we != cudaSuccess) return cuda_fail("view: cannot order after the object's writer", we);
-    for (uint32_t pg : o->pages) deps_.mark_read(pg, StreamDeps::kOpen);
+    for (uint32_t pg : o->pages) deps_.mark_view(pg);
     *ptr = reinterpret_cast<void*>(pool_ + (uint64_t(o->pages[0]) << page_shift_));
     return T2I_OK;
 }

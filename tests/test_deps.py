@@ -45,7 +45,7 @@ int main(int argc, char** argv) {
         d.begin(d.stream_index(st));
         if (verb == 'p') d.writes(0); else d.reads(0);
         d.wait();
-        if (verb == 'v') { d.mark_read(0, t2i::StreamDeps::kOpen); return; }
+        if (verb == 'v') { d.mark_view(0); return; }
         st->work++;
         uint32_t q = 0;
         d.end(&q);
