@@ -14,6 +14,7 @@ import numpy as np
 
 from . import _lib as L
 
+_ndarray = np.ndarray
 PUT_DTYPE = np.dtype([("src", "<u8"), ("nbytes", "<u8"), ("src_is_host", "<u4"), ("dtype_tag", "<u4"),
                       ("group", "<u8"), ("order", "<u4"), ("evictable", "<u4"), ("consumers", "<u4"),
                       ("reserved", "<u4")])
@@ -288,14 +289,16 @@ class Store:
         if self._fast is not None:
             if ids is None:
                 return self._fast.get_batch(self._hi, p.addr, p.n, p.out_addr, _stream(stream))
-            if isinstance(ids, np.ndarray):
-                s = _stream(stream)
+            s = _stream(stream)
+            if type(ids) is _ndarray:
                 st = self._fast.get_batch_for(self._hi, p.addr, p.n, ids, p.out_addr, s)
                 if st is not None:
                     return st
-                # an array whose buffer does not say plain uint64 (it is not aligned)
-                if ids.dtype == np.uint64 and ids.flags.c_contiguous and len(ids) >= p.n and ids.size >= p.n:
-                    return self._fast.get_batch_ids(self._hi, p.addr, p.n, ids.ctypes.data, p.out_addr, s)
+            # an array whose buffer does not say plain uint64 (it is not aligned), or of a subclass
+            if (isinstance(ids, np.ndarray) and ids.dtype == np.uint64 and ids.flags.c_contiguous
+                    and len(ids) >= p.n and ids.size >= p.n):
+                return self._fast.get_batch_ids(self._hi, p.addr, p.n, ids.ctypes.data, p.out_addr, s)
+            stream = s
         if ids is not None:
             p.descs["id"] = ids
         return self._lib.t2i_get_batch(self._h, p.addr, p.n, p.out_addr, _stream(stream))
