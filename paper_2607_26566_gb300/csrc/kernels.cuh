@@ -90,13 +90,15 @@ constexpr unsigned kTileMaxPerSm = T2I_TUNE_TILE_BALANCE ? 8 : 0;
 constexpr unsigned kTileOverlapThreads = 320;
 // Such launches of fewer bytes run as warp tiles: of 11.5 MB on four streams,
 // issued from C, 6.82 TB/s, against 6.85 / 6.70 / 6.66 / 6.55 in CTA tiles of 512
-// / 384 / 320 / 256 threads. Above the line, in warp tiles and in CTA tiles of 320
-// threads (us a pass): eight requests put on one stream and got on another, each
-// get waiting for its put, of 14 MiB 124.7 and 117.2, of 16 130.7 and 125.7, of 18
-// 149.2 and 132.8 (there a warp CTA of 31 warps takes an SM's registers); sixteen
-// handoffs on four streams, of 14 MiB 139.0 and 139.9, of 16 164.7 and 158.2, of
-// 18 176.3 and 176.2.
-constexpr uint64_t kTileOverlapMinBytes = 13ull << 20;
+// / 384 / 320 / 256 threads. In warp tiles and in CTA tiles of 320 threads (us a
+// pass): sixteen handoffs on four streams, in scattered 64 KiB pages, of 14 MiB
+// 158.6 and 162.5, of 16 172.1 and 175.3, of 17 175.8 and 176.0, of 19 191.6 and
+// 190.1; in 2 MiB pages of 14 139.0 and 139.9, of 16 164.7 and 158.2, of 18 176.3
+// and 176.2. Eight requests put on one stream and got on another, each get
+// waiting for its put, of 14 MiB 124.7 and 117.2, of 16 130.7 and 125.7, of 18
+// 149.2 and 132.8 (there a warp CTA of 31 warps takes an SM's registers; the
+// kernels before the tiles took 132.1, 134.0 and 140.0).
+constexpr uint64_t kTileOverlapMinBytes = 16ull << 20;
 // Vectors per thread, and the most threads of a kernel of V vectors.
 constexpr int tile_vec(unsigned threads) { return threads >= 512 ? 2 : 4; }
 template <int V>

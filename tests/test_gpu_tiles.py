@@ -131,7 +131,7 @@ def test_gather_without_a_store_overlapping_and_captured():
 
 
 @pytest.mark.parametrize("P", [16384, 65536, 1 << 20])
-@pytest.mark.parametrize("n", [(4 << 20) + 20, (13 << 20) - 16, (13 << 20) + 20, (20 << 20) - 16, (20 << 20) + 20,
+@pytest.mark.parametrize("n", [(4 << 20) + 20, (16 << 20) - 16, (16 << 20) + 20, (20 << 20) - 16, (20 << 20) + 20,
                                (48 << 20) + 4])
 def test_large_calls_on_two_streams_in_turn(P, n):
     """Calls whose launches are shaped to run beside other streams' (and the
