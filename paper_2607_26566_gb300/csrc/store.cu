@@ -1001,7 +1001,7 @@ constexpr uint64_t kNoAllocMaxPagesPerLaunch = (kBlobLarge - sizeof(TileSeg)) / 
 uint64_t noalloc_pages_per_launch(uint64_t page_bytes) {
     return std::min<uint64_t>(kNoAllocMaxPagesPerLaunch, std::max<uint64_t>(1, (uint64_t(1) << 36) / page_bytes));
 }
-constexpr int kNoAllocMaxDevices = 64;
+constexpr int kNoAllocMaxDevices = 64;  // higher device numbers are refused, likewise
 }  // namespace
 }  // namespace t2i
 
