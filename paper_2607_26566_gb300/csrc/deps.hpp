@@ -33,11 +33,13 @@ class StreamDeps {
     struct PageDeps {
         Dep writer;
         Dep readers[2];
-        uint8_t more_readers = 0;  // > 2 reading streams since the last write (2: a view may be among the others)
+        uint8_t more_readers = 0;  // > 2 reading streams since the last write
+        uint16_t viewer = 0;       // stream + 1 that was given a view since (kViewers: several)
     };
+    static constexpr uint16_t kViewers = 0xFFFF;
     static constexpr uint32_t kRing = 64;
-    // a reader whose reads are not calls of the store (a view): later
-    // writers wait for everything its stream has been given by then
+    // a view's reads are not calls of the store: later writers wait for
+    // everything its stream has been given by then
     static constexpr uint32_t kOpen = 0xFFFFFFFFu;
 
     ~StreamDeps() { release(); }
@@ -75,7 +77,7 @@ class StreamDeps {
         since_change_ = si != cur_ ? 0 : since_change_ < kInterleave ? since_change_ + 1 : kInterleave;
         cur_ = si;
         need_.assign(streams_.size(), 0);
-        wait_all_ = 0;
+        wait_all_ = wait_views_ = false;
     }
     void reads(uint32_t page) { note(pages_[page].writer); }
     void writes(uint32_t page) {
@@ -83,7 +85,11 @@ class StreamDeps {
         note(d.writer);
         note(d.readers[0]);
         note(d.readers[1]);
-        if (wait_all_ < d.more_readers) wait_all_ = d.more_readers;
+        if (d.more_readers) wait_all_ = true;
+        if (d.viewer == kViewers)
+            wait_views_ = true;
+        else if (d.viewer)
+            note({kOpen, static_cast<uint16_t>(d.viewer - 1)});
     }
     // Makes the call's stream wait for what it depends on.
     cudaError_t wait() {
@@ -91,7 +97,7 @@ class StreamDeps {
         for (size_t j = 0; j < streams_.size(); ++j) {
             uint32_t q = need_[j];
             if (wait_all_ && q < streams_[j].seq) q = streams_[j].seq;
-            if (wait_all_ == 2 && streams_[j].viewed) q = kOpen;
+            if (wait_views_ && streams_[j].viewed) q = kOpen;
             if (int(j) == cur_ || q == 0) continue;
             cudaError_t e = wait_for(static_cast<int>(j), q, s);
             if (e != cudaSuccess) return e;
@@ -118,33 +124,26 @@ class StreamDeps {
         d.writer = {seq, static_cast<uint16_t>(cur_)};
         d.readers[0] = d.readers[1] = Dep{};
         d.more_readers = 0;
+        d.viewer = 0;
     }
     void mark_read(uint32_t page, uint32_t seq) {
         PageDeps& d = pages_[page];
+        const Dep me{seq, static_cast<uint16_t>(cur_)};
         for (Dep& r : d.readers) {
-            if (r.seq == 0) {
-                r = {seq, static_cast<uint16_t>(cur_)};
-                return;
-            }
-            if (r.stream == cur_) {
-                // a view lasts until the page is written: the stream's later
-                // calls do not end its reads
-                if (r.seq != kOpen) r.seq = seq;
+            if (r.seq == 0 || r.stream == me.stream) {
+                r = me;
                 return;
             }
         }
-        if (d.more_readers == 0) d.more_readers = 1;
+        d.more_readers = 1;
     }
+    // A view lasts until the page is written: calls made meanwhile, on its
+    // stream or on others, do not end its reads.
     void mark_view(uint32_t page) {
         PageDeps& d = pages_[page];
+        const uint16_t me = static_cast<uint16_t>(cur_ + 1);
+        d.viewer = d.viewer == 0 || d.viewer == me ? me : kViewers;
         streams_[cur_].viewed = true;
-        for (Dep& r : d.readers) {
-            if (r.seq == 0 || r.stream == cur_) {
-                r = {kOpen, static_cast<uint16_t>(cur_)};
-                return;
-            }
-        }
-        d.more_readers = 2;
     }
 
     // Waits on the host for everything every known stream has been given.
@@ -206,7 +205,8 @@ class StreamDeps {
     std::vector<uint32_t> need_;
     int cur_ = 0;
     uint32_t since_change_ = kInterleave;  // calls since the last change of stream
-    uint8_t wait_all_ = 0;  // the call overwrites a page with more_readers
+    bool wait_all_ = false;    // the call overwrites a page with more_readers
+    bool wait_views_ = false;  // ... or with views on several streams
 };
 
 }  // namespace t2i

@@ -91,6 +91,8 @@ def waited(driver, calls):
     ("vA gB gC kA pD", [1, 1, 1]),              # the view in an entry, more readers than entries
     ("gA gB vC kC kC pD", [1, 1, 2]),           # the view beyond the entries
     ("vA gB gC kA gA kA pD", [3, 1, 1]),
+    ("vA vB vA kA kB kB pB", [1, 0, 0]),        # views on two streams, one of them the writer's
+    ("vA vB kA kB kB pA vC kC pB", [2, 0, 1]),  # a write ends them all
     ("gD gA gB gC kA kB kC pD", [1, 1, 1]),     # without a view: the calls, not the work after them
     ("vA kA pA gB pB kA gB gC gA gD kA pD", [4, 3, 1]),  # a write ends the views before it
 ])
